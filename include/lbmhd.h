@@ -150,9 +150,11 @@ int lbmhd_init(lbmhd_t* h, const double* rho, const double* ux, const double* uy
 int lbmhd_init_device(lbmhd_t* h, const double* rho, const double* ux, const double* uy,
                       const double* bx, const double* by);
 
-/* Advance n >= 0 time steps: each is one fused launch of pull-stream and
- * collide (Sec. 1.2 and Sec. 3) over the whole lattice.  Asynchronous on
- * the handle's stream; long runs replay a captured CUDA graph.  Returns
+/* Advance n >= 0 time steps of fused pull-stream and collide (Sec. 1.2 and
+ * Sec. 3) over the whole lattice, one per launch; FP32 and FP16 storage with
+ * les 0 or 1 advance up to four per launch where steps follow each other
+ * (the same bits; not after lbmhd_set_launch).  Asynchronous on the handle's
+ * stream; long runs replay a captured CUDA graph.  Returns
  * ESTATE before init.  A pending non-finite report (check_finite_every)
  * is returned by the next synchronising call. */
 int lbmhd_step(lbmhd_t* h, int n);
@@ -275,7 +277,8 @@ int64_t lbmhd_launch_count(const lbmhd_t* h);
  * nodes in 32-thread blocks (FP16 storage) or 2 nodes in 128-thread blocks
  * (FP64), falling back to narrower vectors when nx is not a multiple.
  * Results do not depend on the shape (bit for bit).  EINVAL if the shape
- * is not available.
+ * is not available.  A shape that was set is used for every step; without
+ * one, lbmhd_step takes several steps per launch where it can.
  * For les 2 and 3 (steps that need moment gradients): vec = 1 selects the
  * fused kernel (one launch per step; CTAs sweep column strips; `block`
  * ignored on input, reported as strip width + 32), vec = 0 the two-pass

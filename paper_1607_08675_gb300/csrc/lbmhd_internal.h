@@ -55,6 +55,14 @@ cudaError_t launch_step(int prec, int vec, int block, int max_blocks, const void
                         int y1 = -1);
 bool step_variant_ok(int prec, int vec, int nx);
 
+// `steps` (2 .. kPipeSteps) time steps in one pass, src -> dst
+// (lbmhd_step_pipe.cu): the bits of as many launch_step calls.  pipe_ok: the
+// storage format has the kernel and the lattice is large enough for it.
+constexpr int kPipeSteps = 4;
+bool pipe_ok(int prec, const Geom& g);
+cudaError_t launch_pipe(int prec, int steps, const void* src, void* dst, const Geom& g,
+                        const HostColl& c, int sm_count, cudaStream_t st);
+
 // TMA-staged step (lbmhd_step_tma.cu): W threads = nodes per row tile,
 // persistent grid of `grid` CTAs; a timed-out wait sets bit 2 of *status.
 bool tma_variant_ok(int prec, int W, int nx);
@@ -144,8 +152,9 @@ struct lbmhd_t {
     int* d_flag;
     int vec, block;   // register kernel: nodes per thread, threads per block
     int tma_w;        // > 0: TMA-staged kernel with this tile width
+    int pipe;         // several steps per pass (lbmhd_step_pipe.cu) where steps follow each other
     int kin_two_pass; // les 2, 3: moments pass + step instead of the fused kernel
     int sm_count;
     cudaGraphExec_t graph;
-    int graph_steps;
+    int graph_steps, graph_launches;
 };

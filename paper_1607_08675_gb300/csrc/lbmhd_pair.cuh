@@ -1,0 +1,146 @@
+// lbmhd_pair.cuh -- the FP32 collision with every rounding written out, of one
+// node (T = float) or of two neighbouring nodes at once (T = float2) in the
+// packed two-wide FP32 instructions of sm_100 and later, which take one issue
+// slot for two operations.
+//
+// The operations, their order and the fused multiply-adds are those that
+// collide<float> (lbmhd_device.cuh) compiles to in the one-step kernels, so
+// both give the same bits; they were settled by comparing the two over random
+// states, bit for bit.  ABS: FP32 storage of the populations themselves,
+// where the compiler fuses the second product of j_x j_y / rho - B_x B_y
+// instead of the first.  A sign moved from a term to a constant (n8, the
+// outputs, -1/tau_m) changes no rounding.
+#pragma once
+
+#include <type_traits>
+
+#include "lbmhd_device.cuh"
+
+namespace lbmhd {
+
+// One operation on one node (float) or on two (float2), each rounded on its own.
+template <class T>
+__device__ __forceinline__ T dup(float v) {
+    if constexpr (std::is_same<T, float>::value) return v;
+    else return make_float2(v, v);
+}
+__device__ __forceinline__ float add_(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ float sub_(float a, float b) { return __fsub_rn(a, b); }
+__device__ __forceinline__ float mul_(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ float fma_(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ float neg_(float a) { return -a; }
+__device__ __forceinline__ float abs_(float a) { return fabsf(a); }
+__device__ __forceinline__ float2 add_(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 mul_(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 fma_(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ float2 sub_(float2 a, float2 b) {
+    float2 r;
+    asm("{\n\t.reg .b64 ra, rb, rc;\n\tmov.b64 ra, {%2, %3};\n\tmov.b64 rb, {%4, %5};\n\t"
+        "sub.rn.f32x2 rc, ra, rb;\n\tmov.b64 {%0, %1}, rc;\n\t}"
+        : "=f"(r.x), "=f"(r.y)
+        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return r;
+}
+__device__ __forceinline__ float2 neg_(float2 v) { return make_float2(-v.x, -v.y); }
+__device__ __forceinline__ float2 abs_(float2 v) { return make_float2(fabsf(v.x), fabsf(v.y)); }
+__device__ __forceinline__ float2 mul_(float k, float2 b) { return mul_(make_float2(k, k), b); }
+__device__ __forceinline__ float2 fma_(float k, float2 b, float2 c) { return fma_(make_float2(k, k), b, c); }
+__device__ __forceinline__ float2 rcp(float2 v) { return make_float2(rcp(v.x), rcp(v.y)); }
+__device__ __forceinline__ float2 sqrt_(float2 v) { return make_float2(sqrt_(v.x), sqrt_(v.y)); }
+
+// See collide() for the moments, rates and equilibria.
+template <class T, bool SCALED, bool ABS>
+__device__ __forceinline__ void collide_r(T (&d)[9], T (&g)[10], const Coll<float>& c) {
+    constexpr float k1_3 = 1.0f / 3.0f, k1_6 = 1.0f / 6.0f, k5_3 = 5.0f / 3.0f;
+    constexpr float k1_12 = 1.0f / 12.0f, k1_20 = 1.0f / 20.0f, k1_180 = 1.0f / 180.0f;
+    const T s56 = add_(d[5], d[6]), s78 = add_(d[7], d[8]);
+    const T e56 = sub_(d[5], d[6]), e13 = sub_(d[1], d[3]), e24 = sub_(d[2], d[4]);
+    const T e87 = sub_(d[8], d[7]);
+    const T dsum9 = add_(add_(add_(add_(d[0], d[1]), add_(d[2], d[3])),
+                                   add_(add_(d[4], d[5]), add_(d[6], d[7]))), d[8]);
+    const T jx = add_(add_(e13, e56), e87);
+    const T jy = sub_(add_(e24, s56), s78);
+    const T rho = SCALED ? fma_(c.inv_s, dsum9, dup<T>(1.0f)) : add_(dup<T>(1.0f), dsum9);
+    const T irho = rcp(rho);
+    const T ux = mul_(jx, irho), uy = mul_(jy, irho);
+    const T bx = add_(add_(add_(g[0], g[2]), add_(g[4], g[6])), g[8]);
+    const T by = add_(add_(add_(g[1], g[3]), add_(g[5], g[7])), g[9]);
+
+    const T dsum = add_(s56, s78);
+    const T m3 = sub_(e56, e87);
+    const T m4 = sub_(add_(d[1], d[3]), add_(d[2], d[4]));
+    const T m5 = add_(fma_(-2.0f, e13, e56), e87);
+    const T m6 = sub_(fma_(-2.0f, e24, s56), s78);
+    const T f0 = mul_(4.0f, d[0]);
+    const T m7 = fma_(4.0f, dsum, fma_(-5.0f, add_(add_(d[1], d[2]), add_(d[3], d[4])), f0));
+    const T m8 = sub_(f0, dsum);
+
+    const T nbx = neg_(bx), njy = neg_(jy);
+    T j2i = mul_(fma_(jx, jx, mul_(jy, jy)), irho);
+    const T q3 = ABS ? fma_(nbx, by, mul_(mul_(jx, jy), irho)) : fma_(mul_(jx, jy), irho, mul_(nbx, by));
+    const T q4 = fma_(by, by, fma_(fma_(jx, jx, mul_(njy, jy)), irho, mul_(nbx, bx)));
+    T E = fma_(ux, by, mul_(uy, nbx));
+    T n3, n4;
+    if (SCALED) {
+        j2i = mul_(c.inv_s, j2i);
+        E = mul_(c.inv_s, E);
+        n3 = fma_(-c.inv_s, q3, m3);
+        n4 = fma_(-c.inv_s, q4, m4);
+    } else {
+        n3 = sub_(m3, q3);
+        n4 = sub_(m4, q4);
+    }
+    const T n5 = add_(m5, jx), n6 = add_(m6, jy);
+    const T t3 = mul_(3.0f, j2i);
+    const T n7 = add_(m7, t3);
+    const T n8 = add_(m8, fma_(-k5_3, dsum9, t3));
+
+    T snu, nsm;
+    if (c.les) {
+        const T Q = sqrt_(fma_(4.0f, mul_(n3, n3), mul_(n4, n4)));
+        const T te2 = add_(dup<T>(c.tn), sqrt_(fma_(mul_(c.k18, Q), irho, dup<T>(c.tn2))));
+        snu = rcp(mul_(0.5f, te2));
+        const T J = abs_(fma_(-2.0f, E, sub_(sub_(g[3], g[7]), sub_(g[4], g[8]))));
+        const T tm2 = add_(dup<T>(c.te), sqrt_(fma_(c.k36, J, dup<T>(c.te2))));
+        nsm = rcp(mul_(-0.5f, tm2));
+    } else {
+        snu = dup<T>(rcp(c.tn));
+        nsm = dup<T>(rcp(-c.te));
+    }
+    const T s7 = c.s7 > 0.0f ? dup<T>(c.s7) : snu;
+    const T s8 = c.s8 > 0.0f ? dup<T>(c.s8) : snu;
+
+    const T a3 = mul_(0.25f, mul_(snu, n3));
+    const T p4 = mul_(snu, n4), a4 = mul_(0.25f, p4), na4 = mul_(-0.25f, p4);
+    const T a5 = mul_(k1_12, mul_(c.s5, n5));
+    const T a6 = mul_(k1_12, mul_(c.s6, n6));
+    const T a7 = mul_(k1_180, mul_(s7, n7));
+    const T a8 = mul_(k1_20, mul_(s8, n8));
+    const T q78 = sub_(mul_(4.0f, a7), a8);
+    d[0] = fma_(-4.0f, add_(a7, a8), d[0]);
+    d[1] = add_(d[1], fma_(5.0f, a7, fma_(2.0f, a5, na4)));
+    d[2] = add_(d[2], fma_(5.0f, a7, fma_(2.0f, a6, a4)));
+    d[3] = add_(d[3], fma_(5.0f, a7, fma_(-2.0f, a5, na4)));
+    d[4] = add_(d[4], fma_(5.0f, a7, fma_(-2.0f, a6, a4)));
+    const T D = sub_(a3, a5), H = sub_(a6, q78);
+    d[5] = sub_(d[5], add_(add_(a3, a5), add_(a6, q78)));
+    d[6] = sub_(d[6], sub_(sub_(a6, a3), sub_(a5, q78)));
+    d[7] = sub_(d[7], sub_(D, H));
+    d[8] = add_(d[8], add_(D, H));
+
+    const T yp = fma_(3.0f, E, by), xm = fma_(-3.0f, E, bx);
+    const T ym = fma_(-3.0f, E, by), xp = fma_(3.0f, E, bx);
+    auto relax = [&](int q, float k, T v) { g[q] = fma_(nsm, fma_(-k, v, g[q]), g[q]); };
+    relax(0, k1_3, bx);
+    relax(1, k1_3, by);
+    relax(2, k1_6, bx);
+    relax(3, k1_6, yp);
+    relax(4, k1_6, xm);
+    relax(5, k1_6, by);
+    relax(6, k1_6, bx);
+    relax(7, k1_6, ym);
+    relax(8, k1_6, xp);
+    relax(9, k1_6, by);
+}
+
+}  // namespace lbmhd

@@ -1,6 +1,7 @@
 // lbmhd_runtime.cu -- the C ABI of include/lbmhd.h: handle lifetime,
 // parameter validation, buffers, stream-ordered transfers, CUDA-graph
 // replay of long step sequences, error reporting.
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <new>
@@ -152,13 +153,20 @@ cudaError_t launch_one(lbmhd_t* h, const void* src, void* dst) {
     return launch_step(h->p.precision, h->vec, h->block, 0, src, dst, h->geom, h->coll, h->stream);
 }
 
-cudaError_t one_step(lbmhd_t* h) {
-    cudaError_t e = launch_one(h, h->buf[h->cur], h->buf[1 - h->cur]);
-    if (e == cudaSuccess) {
-        h->cur = 1 - h->cur;
-        h->launches += h->coll.kin && h->kin_two_pass ? 2 : 1;
-    }
-    return e;
+// Steps of the next launch when `left` steps follow each other: the passes
+// of at most kPipeSteps steps are kept even (5 = 3 + 2, 6 = 3 + 3), so that
+// only a single step on its own takes the one-step kernel.
+int next_steps(const lbmhd_t* h, int left) {
+    if (!h->pipe || left < 2) return 1;
+    const int passes = (left + kPipeSteps - 1) / kPipeSteps;
+    return (left + passes - 1) / passes;
+}
+
+// One launch of k steps from src to dst.
+cudaError_t launch_steps(lbmhd_t* h, int k, const void* src, void* dst) {
+    if (k > 1)
+        return launch_pipe(h->p.precision, k, src, dst, h->geom, h->coll, h->sm_count, h->stream);
+    return launch_one(h, src, dst);
 }
 
 }  // namespace
@@ -264,6 +272,7 @@ int lbmhd_create(int nx, int ny, const lbmhd_params* p, lbmhd_t** out) {
         }
     h->block = h->vec == 8 ? 32 : (h->vec == 4 ? 64 : (p->precision == LBMHD_FF ? 256 : 128));
     h->tma_w = 0;
+    h->pipe = h->coll.kin == 0 && pipe_ok(p->precision, h->geom);
     // Kinetic steps: the fused kernel where it is faster (measured at 8192^2
     // / 4096^2, MLUPS fused vs two-pass: FP32 les 2 33.5K vs 23.7K, les 3
     // 37.1K vs 22.3K; FP16 38.9K vs 26.6K; FF les 3 8.2K vs 7.2K), the
@@ -301,6 +310,7 @@ int lbmhd_set_launch(lbmhd_t* h, int vec, int block) {
         h->block = block;
         h->tma_w = 0;
     }
+    h->pipe = 0;  // the shape that was asked for, one step per launch
     if (h->graph) cudaGraphExecDestroy(h->graph);
     h->graph = nullptr;
     return LBMHD_OK;
@@ -402,14 +412,19 @@ int lbmhd_step(lbmhd_t* h, int n) {
             if (!h->graph) {
                 cudaGraph_t g = nullptr;
                 LBMHD_CK(h, cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal));
-                for (int s = 0; s < kGraphSteps; ++s) {
-                    const int a = s & 1;
-                    cudaError_t e = launch_one(h, h->buf[a], h->buf[1 - a]);
+                h->graph_launches = 0;
+                int at = 0, done_steps = 0;
+                while (done_steps < kGraphSteps) {
+                    const int k = next_steps(h, kGraphSteps - done_steps);
+                    cudaError_t e = launch_steps(h, k, h->buf[at], h->buf[1 - at]);
                     if (e != cudaSuccess) {
                         cudaStreamEndCapture(h->stream, &g);
                         if (g) cudaGraphDestroy(g);
                         return cuda_fail(h, e, "launch_step (capture)");
                     }
+                    done_steps += k;
+                    at = 1 - at;
+                    ++h->graph_launches;
                 }
                 LBMHD_CK(h, cudaStreamEndCapture(h->stream, &g));
                 cudaError_t e = cudaGraphInstantiate(&h->graph, g, 0);
@@ -418,14 +433,19 @@ int lbmhd_step(lbmhd_t* h, int n) {
                 h->graph_steps = kGraphSteps;
             }
             LBMHD_CK(h, cudaGraphLaunch(h->graph, h->stream));
-            h->launches += kGraphSteps * (h->coll.kin && h->kin_two_pass ? 2 : 1);
+            h->launches += h->graph_launches * (h->coll.kin && h->kin_two_pass ? 2 : 1);
             done += kGraphSteps;
             h->steps += kGraphSteps;
             continue;
         }
-        LBMHD_CK(h, one_step(h));
-        ++done;
-        ++h->steps;
+        // steps up to the next finiteness check follow each other
+        const int run = every > 0 ? std::min<int64_t>(left, every - h->steps % every) : left;
+        const int k = next_steps(h, run);
+        LBMHD_CK(h, launch_steps(h, k, h->buf[h->cur], h->buf[1 - h->cur]));
+        h->cur = 1 - h->cur;
+        h->launches += h->coll.kin && h->kin_two_pass ? 2 : 1;
+        done += k;
+        h->steps += k;
         if (every > 0 && h->steps % every == 0)
             LBMHD_CK(h, launch_check_finite(h->p.precision, h->buf[h->cur], h->d_flag, h->geom,
                                             h->coll, h->stream));

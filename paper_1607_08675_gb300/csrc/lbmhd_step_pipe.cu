@@ -1,0 +1,337 @@
+// lbmhd_step_pipe.cu -- S = 2, 3 or 4 LB-MHD time steps in one pass over the
+// state, for the FP32 and FP16 storage forms with the local rates or no
+// closure (les 0, 1): the bits of S single steps (lbmhd_step.cu).
+//
+// Why: the one-step kernel moves 152 B per node update (FP32) at the copy
+// bandwidth (1.03 of it at 8192^2), so only fewer passes over HBM make it
+// faster.  A step is a 3 x 3 stencil, so S steps of a strip of columns need
+// S rows of history and S halo columns on each side, nothing else.
+//
+// How: one warp owns a strip of 64 columns (two neighbouring ones per lane)
+// and a segment of rows, and sweeps down it; no other warp is involved, so
+// there is no barrier and nothing to wait for.  When the first step is at
+// row r, the second is at row r - 1, the third at r - 2: a row that a step
+// has just computed is streamed along x by one shuffle per plane with
+// c_x != 0 and feeds the next step at once (planes with c_y < 0), one row
+// later (c_y = 0, kept in shared memory, each lane its own values) or two
+// rows later (c_y > 0, kept in registers).  The strip's outer S columns (the
+// left side rounded up to an even number, so that every lane's pair is
+// aligned) are computed from incomplete neighbours and not stored:
+// neighbouring strips overlap by them, as segments do by 2 (S - 1) rows.
+// Rows and columns wrap periodically at the loads, so nothing else knows of
+// the edges of the lattice.
+//
+// The next row's 19 planes are fetched into shared memory by cp.async while
+// the present one is computed (each lane copies what it reads itself, so its
+// own wait orders it).  The two columns of a lane go through the collision
+// together in packed two-wide FP32 instructions (lbmhd_pair.cuh).
+//
+// Bound: instruction issue (177 instructions per update and thread at
+// S = 3, 47% of the issue slots and 51% of the FMA pipe busy) with the
+// latency of few warps: the history of S - 1 steps takes registers, two to
+// four warps per scheduler.  Measured on GB300, 8192^2, updates per second:
+//   FP32  one-step 45.9 G;  S = 2 82.6 G;  S = 3 121.5 G;  S = 4 127.9 G
+//   FP16  one-step 81.6 G;  S = 2 124 G;   S = 3 132 G;    S = 4 133.9 G
+// and 1024^2 (FP32) 36.9 -> 93.0 G, 1999 x 1201 (odd rows) 34.3 -> 95.6 G.
+// On the way (FP32, S = 3): scalar collision without the fetch ahead 91 G
+// (61% issue, 1.7 of 4.4 cycles per instruction waiting for the row), with
+// it 104 G, packed 108 G, and 120 G once shared memory held only the nine
+// c_y = 0 planes -- L1 takes what shared memory leaves, and it holds the
+// rows in flight; with the largest shared-memory carve-out S = 2 fell to
+// 57 G, and any spilled register costs half the rate.
+#include "lbmhd_cp_async.cuh"
+#include "lbmhd_internal.h"
+#include "lbmhd_pair.cuh"
+#include "lbmhd_step_body.cuh"
+
+namespace lbmhd {
+
+namespace {
+
+// The lattices this kernel is for.  Large: both state buffers together beyond
+// 80 MB, about where they stop fitting in L2 and the one-step kernel falls to
+// the rate of HBM (FP32, us per step, one-step / this: 768^2 10.6 / 10.4,
+// 1024^2 26.0 / 12.2; FP16 1024^2 12.5 / 12.8).  Small: up to 32768 nodes,
+// where a launch is mostly latency and one for four steps takes less than
+// four (FP32 64^2 2.23 / 1.77, 128^2 2.57 / 1.90, 256^2 3.16 / 3.19).
+// Between them the rows that segments share cost as much as the passes save
+// (FP32 512^2 5.8 / 6.3).
+constexpr long long kPipeBytes = 80LL << 20;
+constexpr long long kPipeSmall = 32768;
+
+// A pair of neighbouring columns of one plane, as stored.
+template <int P>
+struct PairOf {
+    using T = float2;
+};
+template <>
+struct PairOf<P_FP16_DEV> {  // column x0 in the low half
+    using T = unsigned;
+};
+
+// The pair that streams in along CX: the values of columns x - CX.  The
+// outer lanes get a wrong value for the missing column: a halo column whose
+// result is not used.
+template <int CX>
+__device__ __forceinline__ float2 stream1(float2 v) {
+    if constexpr (CX == 0) return v;
+    if constexpr (CX > 0) return make_float2(__shfl_up_sync(0xffffffffu, v.y, 1), v.x);
+    return make_float2(v.y, __shfl_down_sync(0xffffffffu, v.x, 1));
+}
+template <int CX>
+__device__ __forceinline__ unsigned stream1(unsigned v) {
+    if constexpr (CX == 0) return v;
+    if constexpr (CX > 0) return __byte_perm(__shfl_up_sync(0xffffffffu, v, 1), v, 0x5432);
+    return __byte_perm(v, __shfl_down_sync(0xffffffffu, v, 1), 0x5432);
+}
+
+// Both columns of a pair through the collision, stored form to stored form.
+template <int P>
+__device__ __forceinline__ void collide_pair(typename PairOf<P>::T (&z)[kPlanes], const Coll<float>& c) {
+    constexpr bool SC = Fmt<P>::kScaled, ABS = P == P_FP32;
+    float2 d[9], g[10];
+#pragma unroll
+    for (int p = 0; p < kPlanes; ++p) {
+        float2 v;
+        if constexpr (P == P_FP16_DEV) v = __half22float2(*reinterpret_cast<const __half2*>(&z[p]));
+        else v = z[p];
+        if (P == P_FP32 && p < 9) v = add_(v, dup<float2>(-plane_rest<float>(p)));
+        if (p < 9) d[p] = v;
+        else g[p - 9] = v;
+    }
+    collide_r<float2, SC, ABS>(d, g, c);
+#pragma unroll
+    for (int p = 0; p < kPlanes; ++p) {
+        float2 v = p < 9 ? d[p] : g[p - 9];
+        if (P == P_FP32 && p < 9) v = add_(v, dup<float2>(plane_rest<float>(p)));
+        if constexpr (P == P_FP16_DEV) {
+            const __half2 h = __float22half2_rn(v);
+            z[p] = *reinterpret_cast<const unsigned*>(&h);
+        } else {
+            z[p] = v;
+        }
+    }
+}
+
+// Place of plane p among the planes that do not move along y.
+__host__ __device__ constexpr int keep_slot(int p) {
+    int n = 0;
+    for (int q = 0; q < p; ++q) n += plane_cy(q) == 0;
+    return n;
+}
+
+template <int S>
+struct PipeShape {
+    static constexpr int kHalo = (S + 1) / 2 * 2;             // columns left of the output
+    static constexpr int kUseful = (64 - kHalo - S) / 2 * 2;  // output columns of a strip
+};
+
+// Warps per scheduler that the registers are cut for (65536 / 128 / warps).
+// FP32: 128 registers at S = 2, 168 at S = 3, 255 at S = 4 (three warps spill
+// there: 72 G); FP16, whose history is packed, 128 at every S.
+__host__ __device__ constexpr int pipe_warps(int prec, int steps) {
+    return prec == P_FP16_DEV || steps == 2 ? 4 : (steps == 3 ? 3 : 2);
+}
+
+// AL: nx is even, so a lane's pair is one aligned word in every row.
+template <int P, int S, bool AL>
+__global__ void __launch_bounds__(32, 4 * pipe_warps(P, S))
+    pipe_kernel(const typename Fmt<P>::S* __restrict__ src, typename Fmt<P>::S* __restrict__ dst,
+                int nx, int ny, long long ps, int strips, int seglen, Coll<float> c) {
+    using T = typename Fmt<P>::S;
+    using Q = typename PairOf<P>::T;
+    constexpr int HL = PipeShape<S>::kHalo, U = PipeShape<S>::kUseful;
+    // cp.async moves 4 or 8 bytes: odd rows of FP16 are loaded directly
+    constexpr bool PF = AL || P != P_FP16_DEV;
+    __shared__ Q pre[PF ? kPlanes : 1][32];  // the fetched row
+    __shared__ Q keep[S - 1][9][32];         // each step's last row, c_y = 0
+    const int lane = threadIdx.x;
+    const int strip = (int)(blockIdx.x % (unsigned)strips), seg = (int)(blockIdx.x / (unsigned)strips);
+    const int y0 = seg * seglen, y1 = min(y0 + seglen, ny);
+    const int x = strip * U - HL + 2 * lane;  // this lane's first column, unwrapped
+    int xa = x % nx;
+    if (xa < 0) xa += nx;
+    const int xb = xa + 1 == nx ? 0 : xa + 1;
+    const bool outa = x >= strip * U && x < strip * U + U && x < nx;
+    const bool outb = outa && x + 1 < nx;
+    // rows r - 1, r, r + 1 of the row r that the first step is at
+    int rm = (y0 - S) % ny, r0, rp;
+    if (rm < 0) rm += ny;
+    r0 = rm + 1 == ny ? 0 : rm + 1;
+    rp = r0 + 1 == ny ? 0 : r0 + 1;
+
+    // the populations that stream along y into row r0 of the lane's columns
+    auto fetch = [&](Q(&z)[kPlanes]) {
+        const unsigned om = (unsigned)rm * (unsigned)nx, o0 = (unsigned)r0 * (unsigned)nx,
+                       op = (unsigned)rp * (unsigned)nx;
+#pragma unroll
+        for (int p = 0; p < kPlanes; ++p) {
+            const unsigned row = plane_cy(p) == 0 ? o0 : (plane_cy(p) > 0 ? om : op);
+            const T* base = src + p * ps;
+            if constexpr (PF) {
+                if (AL) cp_async_small<2 * sizeof(T)>(&pre[p][lane], base + (row + xa));
+                else if constexpr (P != P_FP16_DEV) {
+                    cp_async_small<4>(&pre[p][lane].x, base + (row + xa));
+                    cp_async_small<4>(&pre[p][lane].y, base + (row + xb));
+                }
+            } else if constexpr (P == P_FP16_DEV) {
+                if (AL) z[p] = *reinterpret_cast<const unsigned*>(base + (row + xa));
+                else z[p] = (unsigned)base[row + xa] | (unsigned)base[row + xb] << 16;
+            } else {
+                if (AL) z[p] = *reinterpret_cast<const float2*>(base + (row + xa));
+                else z[p] = make_float2(base[row + xa], base[row + xb]);
+            }
+        }
+        if (PF) cp_async_commit();
+        rm = r0;
+        r0 = rp;
+        rp = rp + 1 == ny ? 0 : rp + 1;
+    };
+    auto stream = [&](Q(&v)[kPlanes]) {
+#pragma unroll
+        for (int p = 0; p < kPlanes; ++p)
+            v[p] = plane_cx(p) == 0 ? v[p] : (plane_cx(p) > 0 ? stream1<1>(v[p]) : stream1<-1>(v[p]));
+    };
+
+    Q h1[S - 1][kPlanes], h2[S - 1][kPlanes];  // c_y > 0: the last row and the one before
+    const int n = y1 - y0 + 2 * (S - 1);
+    unsigned orow = (unsigned)y0 * (unsigned)nx + (unsigned)x;
+    Q z[kPlanes];
+    if (PF) fetch(z);
+#pragma unroll 1
+    for (int it = 0; it < n; ++it) {
+        if (PF) {
+            cp_async_wait<0>();
+#pragma unroll
+            for (int p = 0; p < kPlanes; ++p) z[p] = pre[p][lane];
+            stream(z);
+            if (it + 1 < n) fetch(z);
+        } else {
+            fetch(z);
+            stream(z);
+        }
+        collide_pair<P>(z, c);
+        bool done = false;  // the next step's rows are not there yet
+#pragma unroll
+        for (int k = 1; k < S; ++k) {
+            if (done) continue;
+            stream(z);
+            Q w[kPlanes];
+#pragma unroll
+            for (int p = 0; p < kPlanes; ++p) {
+                if (plane_cy(p) < 0) w[p] = z[p];
+                else if (plane_cy(p) == 0) {
+                    w[p] = keep[k - 1][keep_slot(p)][lane];
+                    keep[k - 1][keep_slot(p)][lane] = z[p];
+                } else {
+                    w[p] = h2[k - 1][p];
+                    h2[k - 1][p] = h1[k - 1][p];
+                    h1[k - 1][p] = z[p];
+                }
+            }
+            if (it < 2 * k) {
+                done = true;
+                continue;
+            }
+            collide_pair<P>(w, c);
+#pragma unroll
+            for (int p = 0; p < kPlanes; ++p) z[p] = w[p];
+        }
+        if (done) continue;
+        if (outa) {
+#pragma unroll
+            for (int p = 0; p < kPlanes; ++p) {
+                T* o = dst + p * ps + orow;
+                if constexpr (P == P_FP16_DEV) {
+                    if (AL) *reinterpret_cast<unsigned*>(o) = z[p];
+                    else {
+                        o[0] = (T)z[p];
+                        if (outb) o[1] = (T)(z[p] >> 16);
+                    }
+                } else {
+                    if (AL) *reinterpret_cast<float2*>(o) = z[p];
+                    else {
+                        o[0] = z[p].x;
+                        if (outb) o[1] = z[p].y;
+                    }
+                }
+            }
+        }
+        orow += (unsigned)nx;
+    }
+}
+
+// Rows per segment, at most 96 (longer ones let neighbouring strips drift
+// apart and their shared columns leave L2: 8192^2, S = 4, 96 rows 127.9 G,
+// 192 rows 124 G).  The time of a launch is its rounds of resident warps
+// times the rows a warp walks (its segment, the 2 (S - 1) rows around it and
+// about one for the start) times the time of a row, which grows with the
+// warps w that share a scheduler as a + b w microseconds (measured: S = 4
+// 1.25 at one warp, 2.05 at two; S = 3 2.39 at three).  Within 3% of the best
+// length of a sweep at 1024^2, 1999 x 1201, 2048^2 and 8192^2, where a length
+// that leaves part of a round empty costs up to 60%.
+template <int P, int S>
+int pipe_seglen(int strips, int ny, int sm_count) {
+    constexpr int kMost = 96;
+    constexpr double a = S == 2 ? 0.8 : (S == 3 ? 0.56 : 0.45), b = S == 2 ? 0.6 : (S == 3 ? 0.61 : 0.8);
+    const double sched = 4.0 * sm_count;
+    const long long resident = 4LL * pipe_warps(P, S) * sm_count;
+    int best = 1;
+    double best_t = 1e300;
+    for (int len = 1; len <= kMost && len <= ny; ++len) {
+        const long long units = (long long)strips * ((ny + len - 1) / len);
+        const long long rounds = units / resident, rest = units % resident;
+        double t = (double)rounds * (a + b * pipe_warps(P, S));
+        if (rest) t += a + b * (rest > sched ? (double)rest / sched : 1.0);
+        t *= len + 2 * (S - 1) + 1;
+        if (t < best_t) {
+            best_t = t;
+            best = len;
+        }
+    }
+    return best;
+}
+
+template <int P, int S, bool AL>
+cudaError_t launch_pipe_t(const void* src, void* dst, const Geom& g, const HostColl& hc, int sm_count,
+                          cudaStream_t st) {
+    using T = typename Fmt<P>::S;
+    const int strips = (g.nx + PipeShape<S>::kUseful - 1) / PipeShape<S>::kUseful;
+    const int seglen = pipe_seglen<P, S>(strips, g.ny, sm_count);
+    const int nseg = (g.ny + seglen - 1) / seglen;
+    pipe_kernel<P, S, AL><<<(unsigned)strips * (unsigned)nseg, 32, 0, st>>>(
+        (const T*)src, (T*)dst, g.nx, g.ny, g.ps, strips, seglen, coll_for_prec<float>(hc, P));
+    return cudaGetLastError();
+}
+
+template <int P>
+cudaError_t launch_pipe_p(int steps, const void* src, void* dst, const Geom& g, const HostColl& c,
+                          int sm_count, cudaStream_t st) {
+    const bool al = g.nx % 2 == 0;
+    switch (steps) {
+        case 2: return (al ? launch_pipe_t<P, 2, true> : launch_pipe_t<P, 2, false>)(src, dst, g, c, sm_count, st);
+        case 3: return (al ? launch_pipe_t<P, 3, true> : launch_pipe_t<P, 3, false>)(src, dst, g, c, sm_count, st);
+        case 4: return (al ? launch_pipe_t<P, 4, true> : launch_pipe_t<P, 4, false>)(src, dst, g, c, sm_count, st);
+    }
+    return cudaErrorInvalidValue;
+}
+
+}  // namespace
+
+bool pipe_ok(int prec, const Geom& g) {
+    if (prec != P_FP32 && prec != P_FP32_DEV && prec != P_FP16_DEV) return false;
+    const long long n = (long long)g.nx * g.ny;
+    return n <= kPipeSmall || 2 * kPlanes * (long long)storage_bytes(prec) * n >= kPipeBytes;
+}
+
+cudaError_t launch_pipe(int prec, int steps, const void* src, void* dst, const Geom& g,
+                        const HostColl& c, int sm_count, cudaStream_t st) {
+    switch (prec) {
+        case P_FP32: return launch_pipe_p<P_FP32>(steps, src, dst, g, c, sm_count, st);
+        case P_FP32_DEV: return launch_pipe_p<P_FP32_DEV>(steps, src, dst, g, c, sm_count, st);
+        case P_FP16_DEV: return launch_pipe_p<P_FP16_DEV>(steps, src, dst, g, c, sm_count, st);
+    }
+    return cudaErrorInvalidValue;
+}
+
+}  // namespace lbmhd

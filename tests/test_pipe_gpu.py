@@ -1,0 +1,88 @@
+"""Several steps per launch (csrc/lbmhd_step_pipe.cu) against single steps.
+
+The kernel performs the operations of the one-step kernel in their order, so
+the states must be equal bit for bit (tolerance zero), whatever the lattice:
+narrower than a strip's halo, at and around the 60, 56 and 2 x 56 columns that
+a strip stores, odd rows, fewer rows than the steps of a launch.
+"""
+import numpy as np
+import pytest
+
+from paper_1607_08675_gb300 import inputs
+
+pytestmark = pytest.mark.gpu
+
+RATES = dict(tau_nu=0.6, tau_eta=0.65, C_S=0.1)
+SMALL = [(1, 1), (2, 1), (1, 7), (3, 5), (55, 3), (56, 4), (57, 2), (60, 9), (61, 97), (112, 96),
+         (113, 193), (64, 64), (130, 67)]
+# beyond 80 MB in two buffers (FP32), odd and even rows, several rounds of warps
+LARGE = [(1999, 301), (300, 2001)]
+
+
+@pytest.fixture(scope="module")
+def L():
+    import torch
+
+    assert torch.cuda.is_available(), "GPU tests need a CUDA device"
+    from paper_1607_08675_gb300 import build, lbmhd
+
+    build.build()
+    return lbmhd
+
+
+def raw(L, shape, fields, prec, les, calls, single):
+    p = L.lbmhd_params_default(precision=prec, les=les, **RATES)
+    h = L.lbmhd_create(*shape, p)
+    try:
+        if single:
+            L.lbmhd_set_launch(h, 1, 64)
+        L.lbmhd_init(h, *fields)
+        for n in calls:
+            L.lbmhd_step(h, n)
+        assert L.lbmhd_step_count(h) == sum(calls)
+        return L.lbmhd_get_state_raw(h), L.lbmhd_launch_count(h)
+    finally:
+        L.lbmhd_destroy(h)
+
+
+@pytest.mark.parametrize("prec", ["fp32", "fp32_dev", "fp16_dev"])
+@pytest.mark.parametrize("shape", SMALL + LARGE)
+def test_several_steps_per_launch_equal_single_steps(L, prec, shape):
+    fields = inputs.orszag_tang(*shape, seed=3, amp=1e-3)
+    # 2, 3 and 4 steps per launch, mixtures of them, and a lone step
+    calls = (2, 3, 4, 5, 7, 1) if shape in SMALL else (4, 6)
+    for les in (1, 0):
+        got, launches = raw(L, shape, fields, prec, les, calls, False)
+        ref, one = raw(L, shape, fields, prec, les, calls, True)
+        assert np.array_equal(got, ref), (shape, les)
+        assert one == sum(calls)
+        if shape in SMALL:
+            assert launches == 8
+
+
+def test_several_steps_per_launch_with_tied_rates_and_graph_replay(L):
+    """Rates s_7, s_8 tied to the local s_nu and a run long enough for graph
+    replay, in calls that leave the buffers in either parity."""
+    shape = (114, 90)
+    fields = inputs.turbulence(*shape, kmin=2, kmax=5, seed=5)
+    ref = raw(L, shape, fields, "fp32", 1, (133,), True)[0]
+    for calls in ((133,), (3, 130), (64, 1, 68)):
+        assert np.array_equal(raw(L, shape, fields, "fp32", 1, calls, False)[0], ref)
+
+
+def test_finiteness_check_between_launches(L):
+    """check_finite_every counts steps, not launches: the check after step 3
+    of a ten-step call sees the state of step 3."""
+    shape = (48, 40)
+    fields = inputs.orszag_tang(*shape, seed=1)
+    p = L.lbmhd_params_default(precision="fp32", check_finite_every=3, **RATES)
+    h = L.lbmhd_create(*shape, p)
+    try:
+        L.lbmhd_init(h, *fields)
+        L.lbmhd_step(h, 10)
+        L.lbmhd_sync(h)
+        got = L.lbmhd_get_state_raw(h)
+        assert L.lbmhd_launch_count(h) == 4  # 3 + 3 + 3 + 1 steps
+    finally:
+        L.lbmhd_destroy(h)
+    assert np.array_equal(got, raw(L, shape, fields, "fp32", 1, (10,), True)[0])
