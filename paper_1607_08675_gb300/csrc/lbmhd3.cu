@@ -37,6 +37,7 @@
 #include "lbmhd_bulk.cuh"
 #include "lbmhd_device.cuh"
 #include "lbmhd_internal.h"
+#include "lbmhd_narrow.cuh"
 #include "lbmhd_step_body.cuh"
 
 namespace lbmhd {
@@ -1076,86 +1077,258 @@ struct Fields7 {
 // the component along the axis is B_a / 6, the others carry +-3 E_ab with
 // E_ab = u_a B_b - B_a u_b.
 template <int P>
+__device__ __forceinline__ void init3_node(const double r, const double (&u)[3], const double (&B)[3],
+                                           typename Fmt3<P>::S* __restrict__ st, long long i,
+                                           long long ps, double s16) {
+    const double bb = B[0] * B[0] + B[1] * B[1] + B[2] * B[2];
+    const double uu = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
+    const double r3 = 3.0 * r, r45 = 4.5 * r, m225 = 2.25 * bb;
+    const double common = -1.5 * r * uu - 0.75 * bb;
+    const double a_abs = r + common, a_dev = (r - 1.0) + common;
+#pragma unroll
+    for (int p = 0; p < kQ; ++p) {
+        const int cx = pcx(p), cy = pcy(p), cz = pcz(p);
+        double cu = 0.0, cb = 0.0;
+        if (cx) {
+            cu += cx > 0 ? u[0] : -u[0];
+            cb += cx > 0 ? B[0] : -B[0];
+        }
+        if (cy) {
+            cu += cy > 0 ? u[1] : -u[1];
+            cb += cy > 0 ? B[1] : -B[1];
+        }
+        if (cz) {
+            cu += cz > 0 ? u[2] : -u[2];
+            cb += cz > 0 ? B[2] : -B[2];
+        }
+        const int cc = cx * cx + cy * cy + cz * cz;
+        double t = r3 * cu + r45 * cu * cu - 4.5 * cb * cb;
+        if (cc) t += m225 * cc;
+        const double w = wq<double>(p);
+        st[p * ps + i] = Fmt3<P>::from_fd(w * (a_abs + t), w * (a_dev + t), p, s16);
+    }
+    const double E3[3] = {3.0 * (u[1] * B[2] - B[1] * u[2]), 3.0 * (u[0] * B[2] - B[0] * u[2]),
+                          3.0 * (u[0] * B[1] - B[0] * u[1])};  // 3 E_yz, 3 E_xz, 3 E_xy
+    const double sixth = 1.0 / 6.0;
+#pragma unroll
+    for (int q = 0; q < kM; ++q) {
+        const int a = q / 2;
+        const double sg = q % 2 ? -1.0 : 1.0;
+#pragma unroll
+        for (int b = 0; b < 3; ++b) {
+            double gv;
+            if (b == a) {
+                gv = sixth * B[b];
+            } else {
+                // E_ab = -E_ba; E3 is indexed by the axis not in {a, b}
+                const double e = (a < b ? 1.0 : -1.0) * E3[3 - a - b];
+                gv = sixth * (B[b] + sg * e);
+            }
+            st[(kQ + 3 * q + b) * ps + i] = Fmt3<P>::from_fd(gv, gv, kQ + 3 * q + b, s16);
+        }
+    }
+}
+template <int P>
+__device__ __noinline__ void init3_node_f64(const double r, const double (&u)[3], const double (&B)[3],
+                                            typename Fmt3<P>::S* __restrict__ st, long long i,
+                                            long long ps, double s16) {
+    init3_node<P>(r, u, B, st, i, ps, s16);
+}
+
+// The same equilibria in double-word FP32 (FP32 and FP16 storage): false where
+// a value's rounding is not settled.  Directions c and -c share every even
+// term.  Error bound as in 2D: fewer than 40 operations of 2^-48, relative to
+// the sum m of the terms' magnitudes.
+template <int P>
+__device__ __forceinline__ bool init3_node_ff(double dr, const double (&du)[3], const double (&dB)[3],
+                                              typename Fmt3<P>::S* __restrict__ st, long long i,
+                                              long long ps, double s16) {
+    bool ok = true, open = false;
+    const ff r = split_f64(dr, ok);
+    ff u[3], B[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        u[a] = split_f64(du[a], ok);
+        B[a] = split_f64(dB[a], ok);
+    }
+    const float au = fabsf(u[0].hi) + fabsf(u[1].hi) + fabsf(u[2].hi);
+    const float ab = fabsf(B[0].hi) + fabsf(B[1].hi) + fabsf(B[2].hi), ar = fabsf(r.hi);
+    const bool unit = P != P_FP32 && __double2hiint(dr) == 0x3ff00000 && __double2loint(dr) == 0;
+    const float m = (P == P_FP32 ? ar : (unit ? 0.0f : ar + 1.0f)) + ar * au * (3.0f + 6.0f * au) + 12.0f * ab * ab;
+    const ff sc = ff(s16);
+    auto put = [&](int p, ff x, float err) {
+        if constexpr (P == P_FP16_DEV) st[p * ps + i] = round_ff_half(x * sc, err * (float)s16, open);
+        else st[p * ps + i] = round_ff(x, err, open);
+    };
+    const ff r45 = kmul(4.5f, r);
+    ff ru3[3], uu[3], BB[3], uv[3], BC[3];  // uv, BC: 2 u_a u_b for (xy, xz, yz)
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        ru3[a] = kmul(3, r * u[a]);
+        uu[a] = u[a] * u[a];
+        BB[a] = B[a] * B[a];
+        const int k = a == 2 ? 1 : 0, l = a == 0 ? 1 : 2;
+        uv[a] = kmul(2, u[k] * u[l]);
+        BC[a] = kmul(2, B[k] * B[l]);
+    }
+    const ff bb = BB[0] + BB[1] + BB[2], m225 = kmul(2.25f, bb);
+    ff a = kmul(-1.5f, r * (uu[0] + uu[1] + uu[2])) - kmul(0.75f, bb);
+    a = (P == P_FP32 ? r : r - ff(1)) + a;
+    ff ac[4];  // with 9/4 B^2 |c|^2
+    ac[0] = a;
+    ac[1] = a + m225;
+    ac[2] = ac[1] + m225;
+    ac[3] = ac[2] + m225;
+#pragma unroll
+    for (int p = 0; p < kQ; ++p) {
+        const int cx = pcx(p), cy = pcy(p), cz = pcz(p);
+        // the first of c and -c, the rest direction included
+        const int lead = cx ? cx : (cy ? cy : cz);
+        if (lead < 0) continue;
+        const ff w = ff(wq<double>(p));
+        const float err = m * (float)wq<double>(p) * 0x1p-41f;
+        if (lead == 0) {
+            put(p, w * a, err);
+            continue;
+        }
+        ff odd, sq, sb;
+        bool first = true;
+        auto take = [&](ff& t, ff x) { t = first ? x : t + x; };
+        if (cx) { take(odd, ru3[0]); take(sq, uu[0]); take(sb, BB[0]); first = false; }
+        if (cy) { take(odd, cy > 0 ? ru3[1] : -ru3[1]); take(sq, uu[1]); take(sb, BB[1]); first = false; }
+        if (cz) { take(odd, cz > 0 ? ru3[2] : -ru3[2]); take(sq, uu[2]); take(sb, BB[2]); first = false; }
+        if (cx && cy) { sq += cx * cy > 0 ? uv[0] : -uv[0]; sb += cx * cy > 0 ? BC[0] : -BC[0]; }
+        if (cx && cz) { sq += cx * cz > 0 ? uv[1] : -uv[1]; sb += cx * cz > 0 ? BC[1] : -BC[1]; }
+        if (cy && cz) { sq += cy * cz > 0 ? uv[2] : -uv[2]; sb += cy * cz > 0 ? BC[2] : -BC[2]; }
+        const ff base = ac[cx * cx + cy * cy + cz * cz] + (r45 * sq - kmul(4.5f, sb));
+        // the plane of -c: each 1D index 1 <-> 2
+        const int o = (cz ? 3 - p / 9 : 0) * 9 + (cy ? 3 - p / 3 % 3 : 0) * 3 + (cx ? 3 - p % 3 : 0);
+        put(p, w * (base + odd), err);
+        put(o, w * (base - odd), err);
+    }
+    const ff sixth = ff(1.0 / 6.0);
+    ff B6[3];
+    float eB[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        B6[k] = sixth * B[k];
+        eB[k] = fabsf(B[k].hi) * 0x1p-43f;
+    }
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+#pragma unroll
+        for (int l = k + 1; l < 3; ++l) {
+            const ff E3 = kmul(3, u[k] * B[l] - B[k] * u[l]);  // 3 E_kl
+            const float eE = 3.0f * (fabsf(u[k].hi * B[l].hi) + fabsf(B[k].hi * u[l].hi)) * 0x1p-42f;
+            // axis k, component l: B_l +- 3 E_kl; axis l, component k: B_k -+ 3 E_kl
+            put(kQ + 3 * (2 * k) + l, sixth * (B[l] + E3), eB[l] + eE);
+            put(kQ + 3 * (2 * k + 1) + l, sixth * (B[l] - E3), eB[l] + eE);
+            put(kQ + 3 * (2 * l) + k, sixth * (B[k] - E3), eB[k] + eE);
+            put(kQ + 3 * (2 * l + 1) + k, sixth * (B[k] + E3), eB[k] + eE);
+        }
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        put(kQ + 3 * (2 * k) + k, B6[k], eB[k]);
+        put(kQ + 3 * (2 * k + 1) + k, B6[k], eB[k]);
+    }
+    return ok && !open;
+}
+
+template <int P>
 __global__ void init3_kernel(Fields7 in, long long n, typename Fmt3<P>::S* __restrict__ st,
                              long long ps, double s16) {
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
          i += (long long)gridDim.x * blockDim.x) {
         const double r = in.f[0][i], u[3] = {in.f[1][i], in.f[2][i], in.f[3][i]},
                      B[3] = {in.f[4][i], in.f[5][i], in.f[6][i]};
-        const double bb = B[0] * B[0] + B[1] * B[1] + B[2] * B[2];
-        const double uu = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
-        const double r3 = 3.0 * r, r45 = 4.5 * r, m225 = 2.25 * bb;
-        const double common = -1.5 * r * uu - 0.75 * bb;
-        const double a_abs = r + common, a_dev = (r - 1.0) + common;
-#pragma unroll
-        for (int p = 0; p < kQ; ++p) {
-            const int cx = pcx(p), cy = pcy(p), cz = pcz(p);
-            double cu = 0.0, cb = 0.0;
-            if (cx) {
-                cu += cx > 0 ? u[0] : -u[0];
-                cb += cx > 0 ? B[0] : -B[0];
-            }
-            if (cy) {
-                cu += cy > 0 ? u[1] : -u[1];
-                cb += cy > 0 ? B[1] : -B[1];
-            }
-            if (cz) {
-                cu += cz > 0 ? u[2] : -u[2];
-                cb += cz > 0 ? B[2] : -B[2];
-            }
-            const int cc = cx * cx + cy * cy + cz * cz;
-            double t = r3 * cu + r45 * cu * cu - 4.5 * cb * cb;
-            if (cc) t += m225 * cc;
-            const double w = wq<double>(p);
-            st[p * ps + i] = Fmt3<P>::from_fd(w * (a_abs + t), w * (a_dev + t), p, s16);
-        }
-        const double E3[3] = {3.0 * (u[1] * B[2] - B[1] * u[2]), 3.0 * (u[0] * B[2] - B[0] * u[2]),
-                              3.0 * (u[0] * B[1] - B[0] * u[1])};  // 3 E_yz, 3 E_xz, 3 E_xy
-        const double sixth = 1.0 / 6.0;
-#pragma unroll
-        for (int q = 0; q < kM; ++q) {
-            const int a = q / 2;
-            const double sg = q % 2 ? -1.0 : 1.0;
-#pragma unroll
-            for (int b = 0; b < 3; ++b) {
-                double gv;
-                if (b == a) {
-                    gv = sixth * B[b];
-                } else {
-                    // E_ab = -E_ba; E3 is indexed by the axis not in {a, b}
-                    const double e = (a < b ? 1.0 : -1.0) * E3[3 - a - b];
-                    gv = sixth * (B[b] + sg * e);
-                }
-                st[(kQ + 3 * q + b) * ps + i] = Fmt3<P>::from_fd(gv, gv, kQ + 3 * q + b, s16);
-            }
-        }
+        if constexpr (P == P_FP64 || P == P_FF) init3_node<P>(r, u, B, st, i, ps, s16);
+        else if (!init3_node_ff<P>(r, u, B, st, i, ps, s16)) init3_node_f64<P>(r, u, B, st, i, ps, s16);
     }
 }
 
-// rho, u (3), B (3) of the stored state into seven FP64 fields.
+// rho, u (3), B (3) of one node of the stored state.
+template <int P>
+__device__ __forceinline__ void moments3_node_f64(const typename Fmt3<P>::S* __restrict__ st, long long ps,
+                                                  long long i, double i16, double (&m)[7]) {
+    double rho = 0.0, j[3] = {0.0, 0.0, 0.0}, B[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+    for (int p = 0; p < kQ; ++p) {
+        const double f = Fmt3<P>::to_f(st[p * ps + i], p, i16);
+        rho += f;
+        j[0] += pcx(p) * f;
+        j[1] += pcy(p) * f;
+        j[2] += pcz(p) * f;
+    }
+#pragma unroll
+    for (int q = 0; q < kM; ++q)
+#pragma unroll
+        for (int b = 0; b < 3; ++b)
+            B[b] += Fmt3<P>::to_f(st[(kQ + 3 * q + b) * ps + i], kQ + 3 * q + b, i16);
+    m[0] = rho;
+    for (int a = 0; a < 3; ++a) {
+        m[1 + a] = j[a] / rho;
+        m[4 + a] = B[a];
+    }
+}
+template <int P>
+__device__ __noinline__ void moments3_node_odd(const typename Fmt3<P>::S* __restrict__ st, long long ps,
+                                               long long i, double i16, double (&m)[7]) {
+    moments3_node_f64<P>(st, ps, i, i16, m);
+}
+
+// The seven fields of every node.  FP32 and FP16 values sum exactly in FP64 in
+// any order: line, plane and volume sums (75 FP64 operations against about
+// 250), widened by moving bits, and one reciprocal.
 template <int P>
 __global__ void moments3_kernel(const typename Fmt3<P>::S* __restrict__ st, long long ps,
                                 long long n, Fields7 out, double i16) {
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
          i += (long long)gridDim.x * blockDim.x) {
-        double rho = 0.0, j[3] = {0.0, 0.0, 0.0}, B[3] = {0.0, 0.0, 0.0};
+        double m[7];
+        if constexpr (P == P_FP32 || P == P_FP16_DEV) {
+            bool odd = false;
+            auto val = [&](int p) {
+                if constexpr (P == P_FP16_DEV) return widen_f32(__half2float(__ushort_as_half(st[p * ps + i])), odd);
+                else return widen_f32(st[p * ps + i], odd);
+            };
+            double pl[3], pjy[3], pjx[3];  // planes k_z: sum, j_y, j_x
 #pragma unroll
-        for (int p = 0; p < kQ; ++p) {
-            const double f = Fmt3<P>::to_f(st[p * ps + i], p, i16);
-            rho += f;
-            j[0] += pcx(p) * f;
-            j[1] += pcy(p) * f;
-            j[2] += pcz(p) * f;
+            for (int kz = 0; kz < 3; ++kz) {
+                double ln[3], lx[3];  // lines k_y
+#pragma unroll
+                for (int ky = 0; ky < 3; ++ky) {
+                    const int p = 9 * kz + 3 * ky;
+                    const double c0 = val(p), cp = val(p + 1), cm = val(p + 2);
+                    ln[ky] = c0 + (cp + cm);
+                    lx[ky] = cp - cm;
+                }
+                pl[kz] = ln[0] + (ln[1] + ln[2]);
+                pjy[kz] = ln[1] - ln[2];
+                pjx[kz] = lx[0] + (lx[1] + lx[2]);
+            }
+            m[0] = pl[0] + (pl[1] + pl[2]);
+            double j[3] = {pjx[0] + (pjx[1] + pjx[2]), pjy[0] + (pjy[1] + pjy[2]), pl[1] - pl[2]}, u[3];
+#pragma unroll
+            for (int b = 0; b < 3; ++b)
+                m[4 + b] = ((val(kQ + b) + val(kQ + 3 + b)) + (val(kQ + 6 + b) + val(kQ + 9 + b))) +
+                           (val(kQ + 12 + b) + val(kQ + 15 + b));
+            if constexpr (P == P_FP16_DEV) {
+                m[0] = __fma_rn(m[0], i16, 1.0);
+#pragma unroll
+                for (int a = 0; a < 3; ++a) {
+                    j[a] *= i16;
+                    m[4 + a] *= i16;
+                }
+            }
+            divide_all<3>(j, m[0], u);
+#pragma unroll
+            for (int a = 0; a < 3; ++a) m[1 + a] = u[a];
+            if (odd) moments3_node_odd<P>(st, ps, i, i16, m);
+        } else {
+            moments3_node_f64<P>(st, ps, i, i16, m);
         }
 #pragma unroll
-        for (int q = 0; q < kM; ++q)
-#pragma unroll
-            for (int b = 0; b < 3; ++b) B[b] += Fmt3<P>::to_f(st[(kQ + 3 * q + b) * ps + i], kQ + 3 * q + b, i16);
-        out.f[0][i] = rho;
-        for (int a = 0; a < 3; ++a) {
-            out.f[1 + a][i] = j[a] / rho;
-            out.f[4 + a][i] = B[a];
-        }
+        for (int q = 0; q < 7; ++q) out.f[q][i] = m[q];
     }
 }
 

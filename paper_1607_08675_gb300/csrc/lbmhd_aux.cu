@@ -4,6 +4,7 @@
 #include "lbmhd_device.cuh"
 #include "lbmhd_diag_plan.h"
 #include "lbmhd_internal.h"
+#include "lbmhd_narrow.cuh"
 
 #include <mutex>
 #include <type_traits>
@@ -38,6 +39,103 @@ __device__ __forceinline__ typename Fmt<P>::S enc_d(double absval, double devval
 }
 
 // ---- equilibrium initialisation (Sec. 3 equilibria) ----------------------
+// One node in FP64: f^eq = w [r (1 - 3/2 u^2) + 3 r c.u + 9/2 r (c.u)^2 +
+// 9/4 B^2 c^2 - 9/2 (c.B)^2]; the deviation f^eq - w replaces r (1 - ...) by
+// (r - 1) - 3/2 r u^2.  g_k^eq = w'_k [B + 3 ((C_k.u) B - (C_k.B) u)]: B/3 at
+// rest; on an axis the component along it is w' B exactly, the other one
+// carries +-3 E with E = u_x B_y - u_y B_x.
+template <int P>
+__device__ __forceinline__ void init_node(double r, double u, double v, double Bx, double By,
+                                          typename Fmt<P>::S* __restrict__ st, long long c,
+                                          long long ps, float scale) {
+    const double u2 = u * u + v * v, b2 = Bx * Bx + By * By;
+    const double r3 = 3.0 * r, r45 = 4.5 * r, m225 = 2.25 * b2, ru2 = 1.5 * r * u2;
+    const double a_abs = r - ru2, a_dev = (r - 1.0) - ru2;
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+        const int cx = plane_cx(i), cy = plane_cy(i);
+        const double cu = cx * u + cy * v, cb = cx * Bx + cy * By;
+        const int c2 = cx * cx + cy * cy;
+        const double w = plane_rest<double>(i);
+        double t = r3 * cu + r45 * cu * cu - 4.5 * cb * cb;
+        if (c2) t += m225 * c2;
+        st[i * ps + c] = enc_d<P>(w * (a_abs + t), w * (a_dev + t), scale);
+    }
+    const double E3 = 3.0 * (u * By - v * Bx);
+    const double third = 1.0 / 3.0, sixth = 1.0 / 6.0;
+    const double gv[10] = {third * Bx,        third * By,          // k = 0
+                           sixth * Bx,        sixth * (By + E3),   // +x
+                           sixth * (Bx - E3), sixth * By,          // +y
+                           sixth * Bx,        sixth * (By - E3),   // -x
+                           sixth * (Bx + E3), sixth * By};         // -y
+#pragma unroll
+    for (int q = 0; q < 10; ++q) st[(9 + q) * ps + c] = enc_d<P>(gv[q], gv[q], scale);
+}
+template <int P>
+__device__ __noinline__ void init_node_f64(double r, double u, double v, double Bx, double By,
+                                           typename Fmt<P>::S* __restrict__ st, long long c,
+                                           long long ps, float scale) {
+    init_node<P>(r, u, v, Bx, By, st, c, ps, scale);
+}
+
+// The same equilibria in double-word FP32, for the FP32 and FP16 forms.  False
+// where a value's rounding is not settled (nothing to rely on was stored).
+// Error bound: fewer than 40 operations of 2^-48 each on the way to a value,
+// relative to the sum m of its terms' magnitudes, so 2^-41 m w.
+template <int P>
+__device__ __forceinline__ bool init_node_ff(double dr, double du, double dv, double dX, double dY,
+                                             typename Fmt<P>::S* __restrict__ st, long long c,
+                                             long long ps, float scale) {
+    bool ok = true, open = false;
+    const ff r = split_f64(dr, ok), u = split_f64(du, ok), v = split_f64(dv, ok),
+             X = split_f64(dX, ok), Y = split_f64(dY, ok);
+    const float au = fabsf(u.hi) + fabsf(v.hi), ab = fabsf(X.hi) + fabsf(Y.hi), ar = fabsf(r.hi);
+    // r - 1 is exact where r is 1: fields at rest keep exact zeros
+    const bool unit = P != P_FP32 && __double2hiint(dr) == 0x3ff00000 && __double2loint(dr) == 0;
+    const float m = (P == P_FP32 ? ar : (unit ? 0.0f : ar + 1.0f)) + ar * au * (3.0f + 6.0f * au) + 9.0f * ab * ab;
+    const float sc = P == P_FP16_DEV ? scale : 1.0f;
+    const ff uu = u * u, vv = v * v, uv = kmul(2, u * v), XX = X * X, YY = Y * Y, XY = kmul(2, X * Y);
+    const ff u2 = uu + vv, b2 = XX + YY;
+    const ff r3u = kmul(3, r * u), r3v = kmul(3, r * v), r45 = kmul(4.5f, r), m225 = kmul(2.25f, b2);
+    const ff a = (P == P_FP32 ? r : r - ff(1)) - kmul(1.5f, r * u2);
+    const ff a1 = a + m225, a2 = a1 + m225;
+    auto put = [&](int p, ff x, float err) {
+        if constexpr (P == P_FP16_DEV) st[p * ps + c] = round_ff_half(x * ff(scale, 0.0f), err * sc, open);
+        else st[p * ps + c] = round_ff(x, err, open);
+    };
+    auto pair = [&](int i, int j, ff base, ff odd) {  // directions c and -c
+        const ff w = ff(plane_rest<double>(i));
+        const float err = m * (float)plane_rest<double>(i) * 0x1p-41f;
+        put(i, w * (base + odd), err);
+        put(j, w * (base - odd), err);
+    };
+    put(0, ff(plane_rest<double>(0)) * a, m * (float)plane_rest<double>(0) * 0x1p-41f);
+    pair(1, 3, a1 + (r45 * uu - kmul(4.5f, XX)), r3u);
+    pair(2, 4, a1 + (r45 * vv - kmul(4.5f, YY)), r3v);
+    pair(5, 7, a2 + (r45 * (u2 + uv) - kmul(4.5f, b2 + XY)), r3u + r3v);
+    pair(8, 6, a2 + (r45 * (u2 - uv) - kmul(4.5f, b2 - XY)), r3u - r3v);
+    const ff E3 = kmul(3, u * Y - v * X);
+    const ff third = ff(1.0 / 3.0), sixth = ff(1.0 / 6.0);
+    // per component, so that one that is zero stays settled
+    const float eX = fabsf(X.hi) * 0x1p-43f, eY = fabsf(Y.hi) * 0x1p-43f;
+    const float eE = 3.0f * (fabsf(u.hi * Y.hi) + fabsf(v.hi * X.hi)) * 0x1p-42f;
+    const ff X6 = sixth * X, Y6 = sixth * Y;
+    put(9, third * X, eX);
+    put(10, third * Y, eY);
+    put(11, X6, eX);
+    put(12, sixth * (Y + E3), eY + eE);
+    put(13, sixth * (X - E3), eX + eE);
+    put(14, Y6, eY);
+    put(15, X6, eX);
+    put(16, sixth * (Y - E3), eY + eE);
+    put(17, sixth * (X + E3), eX + eE);
+    put(18, Y6, eY);
+    return ok && !open;
+}
+
+// FP64 and FF storage in FP64.  The others in double-word FP32, a node whose
+// rounding is not settled there (about one in 3000 of a turbulent field)
+// again in FP64.
 template <int P>
 __global__ void init_kernel(const double* __restrict__ rho, const double* __restrict__ ux,
                             const double* __restrict__ uy, const double* __restrict__ bx,
@@ -47,45 +145,23 @@ __global__ void init_kernel(const double* __restrict__ rho, const double* __rest
     for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < n;
          c += (long long)gridDim.x * blockDim.x) {
         const double r = rho[c], u = ux[c], v = uy[c], Bx = bx[c], By = by[c];
-        if (bad && !(r > 0.0 && isfinite(r))) atomicOr(bad, 8);
-        const double u2 = u * u + v * v, b2 = Bx * Bx + By * By;
-        // f^eq = w [r (1 - 3/2 u^2) + 3 r c.u + 9/2 r (c.u)^2 + 9/4 B^2 c^2
-        //           - 9/2 (c.B)^2]; the deviation f^eq - w replaces r (1 - ...)
-        // by (r - 1) - 3/2 r u^2.  The node terms are formed once (the init is
-        // bound by GB300's FP64 rate).
-        const double r3 = 3.0 * r, r45 = 4.5 * r, m225 = 2.25 * b2, ru2 = 1.5 * r * u2;
-        const double a_abs = r - ru2, a_dev = (r - 1.0) - ru2;
-#pragma unroll
-        for (int i = 0; i < 9; ++i) {
-            const int cx = plane_cx(i), cy = plane_cy(i);
-            const double cu = cx * u + cy * v, cb = cx * Bx + cy * By;
-            const int c2 = cx * cx + cy * cy;
-            const double w = plane_rest<double>(i);
-            double t = r3 * cu + r45 * cu * cu - 4.5 * cb * cb;
-            if (c2) t += m225 * c2;
-            st[i * ps + c] = enc_d<P>(w * (a_abs + t), w * (a_dev + t), scale);
+        if constexpr (P == P_FP64 || P == P_FF) {
+            if (bad && !(r > 0.0 && isfinite(r))) atomicOr(bad, 8);
+            init_node<P>(r, u, v, Bx, By, st, c, ps, scale);
+        } else if (!init_node_ff<P>(r, u, v, Bx, By, st, c, ps, scale)) {
+            if (bad && !(r > 0.0 && isfinite(r))) atomicOr(bad, 8);
+            init_node_f64<P>(r, u, v, Bx, By, st, c, ps, scale);
+        } else if (bad && !(__double2hiint(r) > 0)) {  // finite here: a sign or zero
+            atomicOr(bad, 8);
         }
-        // g_k^eq = w'_k [B + 3 ((C_k.u) B - (C_k.B) u)]: B/3 at rest; on an axis
-        // the component along it is w' B exactly, the other one carries
-        // +-3 E with E = u_x B_y - u_y B_x
-        const double E3 = 3.0 * (u * By - v * Bx);
-        const double third = 1.0 / 3.0, sixth = 1.0 / 6.0;
-        const double gv[10] = {third * Bx,        third * By,          // k = 0
-                               sixth * Bx,        sixth * (By + E3),   // +x
-                               sixth * (Bx - E3), sixth * By,          // +y
-                               sixth * Bx,        sixth * (By - E3),   // -x
-                               sixth * (Bx + E3), sixth * By};         // -y
-#pragma unroll
-        for (int q = 0; q < 10; ++q) st[(9 + q) * ps + c] = enc_d<P>(gv[q], gv[q], scale);
     }
 }
 
 // ---- moments of a stored state ------------------------------------------
 template <int P>
-__device__ __forceinline__ void node_moments(const typename Fmt<P>::S* __restrict__ st,
-                                             long long ps, long long o, float inv_scale,
-                                             double& r, double& u, double& v, double& Bx,
-                                             double& By) {
+__device__ __forceinline__ void node_moments_f64(const typename Fmt<P>::S* __restrict__ st,
+                                                 long long ps, long long o, float inv_scale,
+                                                 double (&m)[5]) {
     double d[9];
 #pragma unroll
     for (int i = 0; i < 9; ++i) d[i] = dev_of<P>(st[i * ps + o], i, inv_scale);
@@ -94,15 +170,70 @@ __device__ __forceinline__ void node_moments(const typename Fmt<P>::S* __restric
     for (int i = 0; i < 9; ++i) drho += d[i];
     const double jx = (d[1] - d[3]) + (d[5] - d[6]) + (d[8] - d[7]);
     const double jy = (d[2] - d[4]) + (d[5] + d[6]) - (d[7] + d[8]);
-    r = 1.0 + drho;  // the rest weights sum to one
-    u = jx / r;
-    v = jy / r;
-    Bx = 0.0;
-    By = 0.0;
+    m[0] = 1.0 + drho;  // the rest weights sum to one
+    m[1] = jx / m[0];
+    m[2] = jy / m[0];
+    m[3] = 0.0;
+    m[4] = 0.0;
 #pragma unroll
     for (int k = 0; k < 5; ++k) {
-        Bx += dev_of<P>(st[(9 + 2 * k) * ps + o], 9 + 2 * k, inv_scale);
-        By += dev_of<P>(st[(10 + 2 * k) * ps + o], 10 + 2 * k, inv_scale);
+        m[3] += dev_of<P>(st[(9 + 2 * k) * ps + o], 9 + 2 * k, inv_scale);
+        m[4] += dev_of<P>(st[(10 + 2 * k) * ps + o], 10 + 2 * k, inv_scale);
+    }
+}
+template <int P>
+__device__ __noinline__ void node_moments_odd(const typename Fmt<P>::S* __restrict__ st,
+                                              long long ps, long long o, float inv_scale,
+                                              double (&m)[5]) {
+    node_moments_f64<P>(st, ps, o, inv_scale, m);
+}
+
+// The FP32 and FP16 forms: sums of 24-bit values are exact in FP64, so their
+// order is free -- shared pair sums, the weights subtracted once, the FP16
+// scale applied to the sums, and the values widened by moving bits: 34 FP64
+// operations (42 for FP16) instead of about 85.
+template <int P>
+__device__ __forceinline__ void node_moments(const typename Fmt<P>::S* __restrict__ st,
+                                             long long ps, long long o, float inv_scale,
+                                             double (&m)[5]) {
+    if constexpr (P == P_FP64 || P == P_FF) {
+        node_moments_f64<P>(st, ps, o, inv_scale, m);
+    } else {
+        double d[kPlanes];
+        bool odd = false;
+#pragma unroll
+        for (int i = 0; i < kPlanes; ++i) {
+            if constexpr (P == P_FP16_DEV) d[i] = widen_f32(__half2float(__ushort_as_half(st[i * ps + o])), odd);
+            else d[i] = widen_f32(st[i * ps + o], odd);
+        }
+        if (odd) {
+            node_moments_odd<P>(st, ps, o, inv_scale, m);
+            return;
+        }
+        const double s56 = d[5] + d[6], e56 = d[5] - d[6], s78 = d[7] + d[8], e87 = d[8] - d[7];
+        double drho = (d[0] + (s56 + s78)) + ((d[1] + d[3]) + (d[2] + d[4]));
+        double j[2] = {(d[1] - d[3]) + (e56 + e87), (d[2] - d[4]) + (s56 - s78)};
+        double bx = ((d[9] + d[11]) + (d[13] + d[15])) + d[17];
+        double by = ((d[10] + d[12]) + (d[14] + d[16])) + d[18];
+        if constexpr (P == P_FP32) {
+            constexpr double w0 = plane_rest<float>(0), w1 = plane_rest<float>(1), w5 = plane_rest<float>(5);
+            drho -= w0 + 4.0 * w1 + 4.0 * w5;
+        }
+        if constexpr (P == P_FP16_DEV) {
+            const double is = (double)inv_scale;
+            drho *= is;
+            j[0] *= is;
+            j[1] *= is;
+            bx *= is;
+            by *= is;
+        }
+        m[0] = 1.0 + drho;  // the rest weights sum to one
+        double uv[2];
+        divide_all<2>(j, m[0], uv);
+        m[1] = uv[0];
+        m[2] = uv[1];
+        m[3] = bx;
+        m[4] = by;
     }
 }
 
@@ -112,13 +243,13 @@ __global__ void moments_kernel(const typename Fmt<P>::S* __restrict__ st, double
                                float inv_scale) {
     for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < n;
          c += (long long)gridDim.x * blockDim.x) {
-        double r, u, v, Bx, By;
-        node_moments<P>(st, ps, c, inv_scale, r, u, v, Bx, By);
-        rho[c] = r;
-        ux[c] = u;
-        uy[c] = v;
-        bx[c] = Bx;
-        by[c] = By;
+        double m[5];
+        node_moments<P>(st, ps, c, inv_scale, m);
+        rho[c] = m[0];
+        ux[c] = m[1];
+        uy[c] = m[2];
+        bx[c] = m[3];
+        by[c] = m[4];
     }
 }
 
