@@ -552,9 +552,11 @@ int lbmhd_batch_create(int nruns, const int* nx, const int* ny, const double* ta
     }
     cudaMemset(b->d_bar, 0, 2 * sizeof(unsigned));
     cudaMemset(b->d_flag, 0, sizeof(int));
-    // default shape: the widest vector dividing every run's nx, 64 threads
+    // default shape: the widest vector dividing every run's nx (one node for
+    // FP64), 64 threads at four nodes, 128 below
     int v = 4;
-    if (common->precision == LBMHD_FP64 || common->precision == LBMHD_FF) v = 2;
+    if (common->precision == LBMHD_FF) v = 2;
+    if (common->precision == LBMHD_FP64) v = 1;  // FP64-pipe bound: the finest split
     for (; v > 1; v >>= 1) {
         bool ok = true;
         for (int r = 0; r < nruns; ++r) ok = ok && nx[r] % v == 0;

@@ -129,6 +129,8 @@ struct Coll {
     R k18, k36;      // 18 C_S Delta^2, 36 C_S Delta^2
     R s5, s6;        // resolved energy-flux rates
     R s7, s8;        // fixed rates (used when > 0), else tied to s_nu
+    R c5, c6, c7, c8;  // s5 / 12, s6 / 12, s7 / 45, s8 / 20 (FP64 step)
+    int fix7, fix8;    // s7 > 0, s8 > 0
     int les;
     int tie5, tie6;  // s5 (s6) is the tied value 1/tau_nu
     R inv_s;         // scaled storage: 1 / scale (k18, k36 already divided by scale)

@@ -255,22 +255,29 @@ int lbmhd_create(int nx, int ny, const lbmhd_params* p, lbmhd_t** out) {
     h->d_diag = (double*)mem[3];
     h->d_flag = (int*)mem[4];
     cudaMemsetAsync(h->d_flag, 0, sizeof(int), h->stream);
-    // Default launch shape, measured on GB300 at 8192^2: four nodes per
-    // thread in 64-thread blocks for FP32 storage (46.0K MLUPS, 1.03x the
-    // measured copy bandwidth), eight nodes (16-byte loads) in 32-thread
-    // blocks for FP16 storage (82.0K MLUPS, 0.92x), two nodes in 128-thread
-    // blocks for FP64 (FP64-pipe bound) and for double-word FF storage;
-    // narrower vectors when nx is not a multiple.
-    const int want = p->precision == LBMHD_FP64 || p->precision == LBMHD_FF
-                         ? 2
-                         : (p->precision == LBMHD_FP16_DEV ? 8 : 4);
+    // Default launch shape, measured on GB300: four nodes per thread in
+    // 64-thread blocks for FP32 storage (8192^2 46.0K MLUPS, 1.03x the measured
+    // copy bandwidth), eight nodes (16-byte loads) in 32-thread blocks for FP16
+    // storage (82.0K, 0.92x).  FP64 is bound by the FP64 pipe, and one node per
+    // thread in 64-thread blocks spreads it best at every size (us per step, two
+    // nodes in 128-thread blocks / this: 64^2 13.2 / 6.6, 256^2 24.4 / 21.6,
+    // 1024^2 303.9 / 295.4).  Double-word FF: two nodes in 256-thread blocks,
+    // but one in 128-thread blocks where the lattice leaves SMs idle (64^2 7.3 /
+    // 3.9, 256^2 8.0 / 6.8, 512^2 22.7 / 20.5, 768^2 51.5 / 52.1).  Narrower
+    // vectors when nx is not a multiple.
+    const bool ff_small = p->precision == LBMHD_FF && (long long)nx * ny <= 1LL << 18;
+    const int want = p->precision == LBMHD_FP64 || ff_small
+                         ? 1
+                         : (p->precision == LBMHD_FF ? 2 : (p->precision == LBMHD_FP16_DEV ? 8 : 4));
     h->vec = 1;
     for (int v = want; v > 1; v >>= 1)
         if (nx % v == 0) {
             h->vec = v;
             break;
         }
-    h->block = h->vec == 8 ? 32 : (h->vec == 4 ? 64 : (p->precision == LBMHD_FF ? 256 : 128));
+    h->block = h->vec == 8 ? 32
+               : h->vec == 4 || p->precision == LBMHD_FP64 ? 64
+               : p->precision == LBMHD_FF && !ff_small ? 256 : 128;
     h->tma_w = 0;
     h->pipe = h->coll.kin == 0 && pipe_ok(p->precision, h->geom);
     // Kinetic steps: the fused kernel where it is faster (measured at 8192^2

@@ -13,6 +13,7 @@
 #pragma once
 
 #include "lbmhd_device.cuh"
+#include "lbmhd_f64.cuh"
 #include "lbmhd_internal.h"
 
 namespace lbmhd {
@@ -193,15 +194,27 @@ __device__ __forceinline__ void step_body(const typename Fmt<P>::S* __restrict__
 #pragma unroll
     for (int k = 0; k < V; ++k) {
         R d[9], g[10];
+        if constexpr (P == P_FP64) {  // the populations themselves
 #pragma unroll
-        for (int i = 0; i < 9; ++i) d[i] = Fmt<P>::dec(raw[i][k], i, inv_scale);
+            for (int i = 0; i < 9; ++i) d[i] = raw[i][k];
 #pragma unroll
-        for (int q = 0; q < 10; ++q) g[q] = Fmt<P>::dec(raw[9 + q][k], 9 + q, inv_scale);
-        collide<R, Fmt<P>::kScaled>(d, g, c);
+            for (int q = 0; q < 10; ++q) g[q] = raw[9 + q][k];
+            collide64(d, g, c);
 #pragma unroll
-        for (int i = 0; i < 9; ++i) raw[i][k] = Fmt<P>::enc(d[i], i, scale);
+            for (int i = 0; i < 9; ++i) raw[i][k] = d[i];
 #pragma unroll
-        for (int q = 0; q < 10; ++q) raw[9 + q][k] = Fmt<P>::enc(g[q], 9 + q, scale);
+            for (int q = 0; q < 10; ++q) raw[9 + q][k] = g[q];
+        } else {
+#pragma unroll
+            for (int i = 0; i < 9; ++i) d[i] = Fmt<P>::dec(raw[i][k], i, inv_scale);
+#pragma unroll
+            for (int q = 0; q < 10; ++q) g[q] = Fmt<P>::dec(raw[9 + q][k], 9 + q, inv_scale);
+            collide<R, Fmt<P>::kScaled>(d, g, c);
+#pragma unroll
+            for (int i = 0; i < 9; ++i) raw[i][k] = Fmt<P>::enc(d[i], i, scale);
+#pragma unroll
+            for (int q = 0; q < 10; ++q) raw[9 + q][k] = Fmt<P>::enc(g[q], 9 + q, scale);
+        }
     }
 
     if (live) {
@@ -230,6 +243,12 @@ __host__ __device__ inline Coll<R> make_coll_t(double tn, double te, double k18,
     c.s6 = (R)s6;
     c.s7 = (R)s7;
     c.s8 = (R)s8;
+    c.c5 = (R)(s5 / 12.0);
+    c.c6 = (R)(s6 / 12.0);
+    c.c7 = (R)(s7 / 45.0);
+    c.c8 = (R)(s8 / 20.0);
+    c.fix7 = s7 > 0.0;
+    c.fix8 = s8 > 0.0;
     c.les = les;
     c.tie5 = tie5;
     c.tie6 = tie6;
