@@ -273,9 +273,9 @@ int64_t lbmhd_launch_count(const lbmhd_t* h);
  * stream row tiles of `block` nodes (128, 256 or 512, dividing nx) through
  * a shared-memory ring filled by bulk asynchronous copies.  vec = 8 is
  * available for FP16 storage (16-byte loads).  Default: the register
- * kernel with 4 nodes per thread in 64-thread blocks (FP32 storage), 8
- * nodes in 32-thread blocks (FP16 storage), 1 node in 64-thread blocks
- * (FP64) or 2 nodes in 256-thread blocks (FF; 1 in 128-thread blocks up to
+ * kernel with 2 nodes per thread in 128-thread blocks (FP32 storage), 8
+ * nodes in 32-thread blocks (FP16 storage; 4 in 64-thread blocks below 2^20
+ * nodes), 1 node in 64-thread blocks (FP64) or 2 nodes in 256-thread blocks (FF; 1 in 128-thread blocks up to
  * 2^18 nodes), falling back to narrower vectors when nx is not a multiple.
  * Results do not depend on the shape (bit for bit).  EINVAL if the shape
  * is not available.  A shape that was set is used for every step; without

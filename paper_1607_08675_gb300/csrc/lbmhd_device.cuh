@@ -60,7 +60,7 @@ template <> struct Fmt<P_FP32_DEV> {
     static __device__ __forceinline__ S enc(R d, int, float) { return d; }
 };
 // FP16: stored = d * scale.  The step kernels keep the scaled value through
-// the collision (see collide<R, true>), so dec/enc here convert only.
+// the collision (see SCALED below), so dec/enc here convert only.
 template <> struct Fmt<P_FP16_DEV> {
     using S = unsigned short;  // raw binary16 bits
     using R = float;
@@ -232,77 +232,43 @@ __device__ __forceinline__ double kfma(float k, double x, double y) {
 // -(tau_m/3) j_z gives |j|; tau_m = (tau_eta + sqrt(tau_eta^2 +
 // 36 C_S Delta^2 J)) / 2 with J = |N_y1 - N_x2 - 2E|.  g <- g - (g - g^eq)/tau_m.
 //
-// SCALED: d and g hold s times the deviations (FP16 storage scale s).  Every
-// linear step is unchanged; the four quadratic terms get one factor 1/s,
-// the density needs the unscaled sum, and 18 C_S Delta^2, 36 C_S Delta^2
-// arrive divided by s (Q and J are scaled).  The outputs stay scaled.
-//
-// KIN: relax towards the filtered equilibria, sh = Delta^2 corrections of
-// M_3, M_4, M_7 = M_8 and N_y1 (in the units of d and g).
-//
-// TAUS: use the relaxation times sh[0] (tau_e) and sh[1] (tau_m) given by
-// the caller (cross-helicity closure) instead of the local Smagorinsky ones.
-template <class R, bool SCALED = false, bool KIN = false, bool TAUS = false>
-__device__ __forceinline__ void collide(R (&d)[9], R (&g)[10], const Coll<R>& c,
-                                        const R* sh = nullptr) {
+// This form is instantiated for the double-word type; FP32 and FP64 have their
+// own (collide_r in lbmhd_pair.cuh, collide64 in lbmhd_f64.cuh), the kinetic
+// closures collide_xf below.  Sums of one tree per moment: shared pair sums run
+// 10% fewer double-word instructions but 2.7% slower.
+template <class R>
+__device__ __forceinline__ void collide(R (&d)[9], R (&g)[10], const Coll<R>& c) {
     // Rational constants, formed at compile time in the arithmetic type.
     constexpr R k1_3 = R(1) / R(3), k1_6 = R(1) / R(6), k5_3 = R(5) / R(3);
     constexpr R k1_12 = R(1) / R(12), k1_20 = R(1) / R(20), k1_180 = R(1) / R(180);
-    // FP64 (its step is bound by the FP64 pipe) takes the moments and the
-    // relaxation from shared pair sums -- a = d5 - d6, b = d8 - d7,
-    // cc = d5 + d6, e = d7 + d8, p = d1 - d3, q = d2 - d4, r = d1 + d3,
-    // t = d2 + d4: 22 sums for rho, j and M_3..M_8 instead of 43, 8% faster
-    // at 8192^2.  The other types keep one sum tree per moment: the shared
-    // form holds more values live (FP16 storage: 146 registers instead of
-    // 128, 9% slower) and measured 2.7% slower for FF.
-    constexpr bool SH = std::is_same<R, double>::value;
-    const R a = d[5] - d[6], b = d[8] - d[7], cc = d[5] + d[6], e = d[7] + d[8];
-    const R p = d[1] - d[3], q = d[2] - d[4], r = d[1] + d[3], t = d[2] + d[4];
-    const R ab = a + b, ce = cc - e, rt = r + t, shd = cc + e, d0s = d[0] + shd;
-    const R dsum9 = SH ? d0s + rt
-                       : ((d[0] + d[1]) + (d[2] + d[3])) + ((d[4] + d[5]) + (d[6] + d[7])) + d[8];
-    const R jx = SH ? p + ab : (d[1] - d[3]) + (d[5] - d[6]) + (d[8] - d[7]);
-    const R jy = SH ? q + ce : (d[2] - d[4]) + (d[5] + d[6]) - (d[7] + d[8]);
-    const R rho = R(1) + (SCALED ? dsum9 * c.inv_s : dsum9);
+    const R dsum9 = ((d[0] + d[1]) + (d[2] + d[3])) + ((d[4] + d[5]) + (d[6] + d[7])) + d[8];
+    const R jx = (d[1] - d[3]) + (d[5] - d[6]) + (d[8] - d[7]);
+    const R jy = (d[2] - d[4]) + (d[5] + d[6]) - (d[7] + d[8]);
+    const R rho = R(1) + dsum9;
     const R irho = rcp(rho);
     const R ux = jx * irho, uy = jy * irho;
     const R bx = (g[0] + g[2]) + (g[4] + g[6]) + g[8];
     const R by = (g[1] + g[3]) + (g[5] + g[7]) + g[9];
 
-    const R dsum = SH ? shd : (d[5] + d[6]) + (d[7] + d[8]);
-    const R m3 = SH ? a - b : (d[5] - d[6]) + (d[7] - d[8]);
-    const R m4 = SH ? r - t : (d[1] + d[3]) - (d[2] + d[4]);
-    const R m5 = SH ? ab - kmul(2, p) : kmul(2, d[3] - d[1]) + (d[5] - d[6]) + (d[8] - d[7]);
-    const R m6 = SH ? ce - kmul(2, q) : kmul(2, d[4] - d[2]) + (d[5] + d[6]) - (d[7] + d[8]);
-    const R m7 = SH ? kmul(4, d0s) - kmul(5, rt)
-                    : kmul(4, d[0]) - kmul(5, (d[1] + d[2]) + (d[3] + d[4])) + kmul(4, dsum);
+    const R dsum = (d[5] + d[6]) + (d[7] + d[8]);
+    const R m3 = (d[5] - d[6]) + (d[7] - d[8]);
+    const R m4 = (d[1] + d[3]) - (d[2] + d[4]);
+    const R m5 = kmul(2, d[3] - d[1]) + (d[5] - d[6]) + (d[8] - d[7]);
+    const R m6 = kmul(2, d[4] - d[2]) + (d[5] + d[6]) - (d[7] + d[8]);
+    const R m7 = kmul(4, d[0]) - kmul(5, (d[1] + d[2]) + (d[3] + d[4])) + kmul(4, dsum);
     const R m8 = kmul(4, d[0]) - dsum;
 
-    R j2i = (jx * jx + jy * jy) * irho;
-    R q3 = jx * jy * irho - bx * by;
-    R q4 = (jx * jx - jy * jy) * irho - bx * bx + by * by;
+    const R j2i = (jx * jx + jy * jy) * irho;
+    const R q3 = jx * jy * irho - bx * by;
+    const R q4 = (jx * jx - jy * jy) * irho - bx * bx + by * by;
     // Ny1 = sum_k C_kx g_ky, Nx2 = sum_k C_ky g_kx; Ny1^eq = E = -Nx2^eq
-    R E = ux * by - uy * bx;
-    if (SCALED) {
-        j2i *= c.inv_s;
-        q3 *= c.inv_s;
-        q4 *= c.inv_s;
-        E *= c.inv_s;
-    }
-    R k7 = R(0);
-    if (KIN) {
-        q3 += sh[0];
-        q4 += sh[1];
-        k7 = sh[2];
-        E += sh[3];
-    }
+    const R E = ux * by - uy * bx;
     const R n3 = m3 - q3;
     const R n4 = m4 - q4;
     const R n5 = m5 + jx;
     const R n6 = m6 + jy;
-    const R n7 = KIN ? (m7 + kmul(3, j2i)) - k7 : m7 + kmul(3, j2i);
-    const R n8 = KIN ? m8 - ((k5_3 * dsum9 - kmul(3, j2i)) + k7)
-                     : m8 - (k5_3 * dsum9 - kmul(3, j2i));
+    const R n7 = m7 + kmul(3, j2i);
+    const R n8 = m8 - (k5_3 * dsum9 - kmul(3, j2i));
 
     R tau_e = c.tn, tau_m = c.te;
     if (c.les) {
@@ -312,10 +278,6 @@ __device__ __forceinline__ void collide(R (&d)[9], R (&g)[10], const Coll<R>& c,
         const R Nx2 = g[4] - g[8];
         const R J = fabs(Ny1 - Nx2 - kmul(2, E));
         tau_m = kmul(0.5f, c.te + sqrt_(c.te2 + c.k36 * J));
-    }
-    if (TAUS) {
-        tau_e = sh[0];
-        tau_m = sh[1];
     }
     const R snu = rcp(tau_e);
     const R s7 = c.s7 > R(0) ? c.s7 : snu;
@@ -330,32 +292,14 @@ __device__ __forceinline__ void collide(R (&d)[9], R (&g)[10], const Coll<R>& c,
 
     const R q78 = kmul(4, a7) - a8;
     d[0] -= kmul(4, a7 + a8);
-    if constexpr (SH) {
-        // the rows of T from shared partial sums: d1, d3 = (a4 - 5 a7) -+ 2 a5;
-        // d2, d4 = -(a4 + 5 a7) -+ 2 a6; d5, d6 = (a6 + q78) +- (a3 + a5);
-        // d7, d8 = (q78 - a6) +- (a3 - a5)
-        const R w5 = kmul(5, a7);
-        const R u13 = a4 - w5, u24 = -(a4 + w5);
-        const R y5 = kmul(2, a5), y6 = kmul(2, a6);
-        const R P = a3 + a5, M = a3 - a5, S = a6 + q78, D = q78 - a6;
-        d[1] -= u13 - y5;
-        d[2] -= u24 - y6;
-        d[3] -= u13 + y5;
-        d[4] -= u24 + y6;
-        d[5] -= P + S;
-        d[6] -= S - P;
-        d[7] -= M + D;
-        d[8] -= D - M;
-    } else {
-        d[1] -= a4 - kmul(2, a5) - kmul(5, a7);
-        d[2] -= -a4 - kmul(2, a6) - kmul(5, a7);
-        d[3] -= a4 + kmul(2, a5) - kmul(5, a7);
-        d[4] -= -a4 + kmul(2, a6) - kmul(5, a7);
-        d[5] -= (a3 + a5) + (a6 + q78);
-        d[6] -= (a6 - a3) - (a5 - q78);
-        d[7] -= (a3 - a5) - (a6 - q78);
-        d[8] -= (a5 - a3) - (a6 - q78);
-    }
+    d[1] -= a4 - kmul(2, a5) - kmul(5, a7);
+    d[2] -= -a4 - kmul(2, a6) - kmul(5, a7);
+    d[3] -= a4 + kmul(2, a5) - kmul(5, a7);
+    d[4] -= -a4 + kmul(2, a6) - kmul(5, a7);
+    d[5] -= (a3 + a5) + (a6 + q78);
+    d[6] -= (a6 - a3) - (a5 - q78);
+    d[7] -= (a3 - a5) - (a6 - q78);
+    d[8] -= (a5 - a3) - (a6 - q78);
 
     const R sm = rcp(tau_m);
     const R third = k1_3, sixth = k1_6;
@@ -369,6 +313,18 @@ __device__ __forceinline__ void collide(R (&d)[9], R (&g)[10], const Coll<R>& c,
     for (int q = 0; q < 10; ++q) g[q] -= sm * (g[q] - geq[q]);
 }
 
+// Flags of the collisions:
+// SCALED: d and g hold s times the deviations (FP16 storage scale s).  Every
+// linear step is unchanged; the four quadratic terms get one factor 1/s,
+// the density needs the unscaled sum, and 18 C_S Delta^2, 36 C_S Delta^2
+// arrive divided by s (Q and J are scaled).  The outputs stay scaled.
+//
+// KIN: relax towards the filtered equilibria, sh = Delta^2 corrections of
+// M_3, M_4, M_7 = M_8 and N_y1 (in the units of d and g).
+//
+// TAUS: use the relaxation times sh[0] (tau_e) and sh[1] (tau_m) given by
+// the caller (cross-helicity closure) instead of the local Smagorinsky ones.
+//
 // The collision of collide() with its products and sums written as explicit
 // fused multiply-adds (fmad, kfma), for kernels compiled without contraction
 // (the kinetic closures' file): there the compiler fuses nothing by itself,
@@ -381,8 +337,11 @@ __device__ __forceinline__ void collide_xf(R (&d)[9], R (&g)[10], const Coll<R>&
                                            const R* sh = nullptr) {
     constexpr R k1_3 = R(1) / R(3), k1_6 = R(1) / R(6), k5_3 = R(5) / R(3);
     constexpr R k1_12 = R(1) / R(12), k1_20 = R(1) / R(20), k1_180 = R(1) / R(180);
-    // FP64 takes the shared pair sums of collide(); the other types the
-    // sum trees (same measurements).
+    // FP64 (bound by the FP64 pipe) takes the moments and the relaxation from
+    // shared pair sums -- a = d5 - d6, b = d8 - d7, cc = d5 + d6, e = d7 + d8,
+    // p = d1 - d3, q = d2 - d4, r = d1 + d3, t = d2 + d4: 22 sums for rho, j and
+    // M_3..M_8 instead of 43.  The other types keep one sum tree per moment: the
+    // shared form holds more values live (FP16 storage 9% slower, FF 2.7%).
     constexpr bool SH = std::is_same<R, double>::value;
     const R a = d[5] - d[6], b = d[8] - d[7], cc = d[5] + d[6], e = d[7] + d[8];
     const R p = d[1] - d[3], q = d[2] - d[4], r = d[1] + d[3], t = d[2] + d[4];

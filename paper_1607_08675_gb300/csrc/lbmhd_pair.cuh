@@ -3,13 +3,13 @@
 // packed two-wide FP32 instructions of sm_100 and later, which take one issue
 // slot for two operations.
 //
-// The operations, their order and the fused multiply-adds are those that
-// collide<float> (lbmhd_device.cuh) compiles to in the one-step kernels, so
-// both give the same bits; they were settled by comparing the two over random
-// states, bit for bit.  ABS: FP32 storage of the populations themselves,
-// where the compiler fuses the second product of j_x j_y / rho - B_x B_y
-// instead of the first.  A sign moved from a term to a constant (n8, the
-// outputs, -1/tau_m) changes no rounding.
+// Both come from the one source below, and every FP32 step kernel calls it, so
+// they give the same bits whatever shape the compiler gives their code.  The
+// operations are those of collide() (lbmhd_device.cuh) with its products fused
+// into the sums that follow.  ABS: FP32 storage of the populations themselves
+// fuses the second product of j_x j_y / rho - B_x B_y instead of the first.  A
+// sign moved from a term to a constant (n8, the outputs, -1/tau_m) changes no
+// rounding.
 #pragma once
 
 #include <type_traits>
@@ -141,6 +141,36 @@ __device__ __forceinline__ void collide_r(T (&d)[9], T (&g)[10], const Coll<floa
     relax(7, k1_6, ym);
     relax(8, k1_6, xp);
     relax(9, k1_6, by);
+}
+
+// A pair of nodes one after the other: for threads with more nodes, where the
+// packed form's live values cost more in occupancy than its issue slots save
+// (us per step, each / packed: FP32 512^2 four nodes 5.9 / 6.5, FP16 512^2 four
+// nodes 4.2 / 5.0, FP16 1024^2 eight nodes 12.5 / 13.4; with two nodes packed
+// wins: FP32 512^2 5.9 / 5.4, 1024^2 27.1 / 23.8, FP16 512^2 5.2 / 4.7).
+template <bool SCALED, bool ABS>
+__device__ __forceinline__ void collide_pair_each(float2 (&d)[9], float2 (&g)[10], const Coll<float>& c) {
+    float a[9], b[10];
+#pragma unroll
+    for (int i = 0; i < 9; ++i) a[i] = d[i].x;
+#pragma unroll
+    for (int q = 0; q < 10; ++q) b[q] = g[q].x;
+    collide_r<float, SCALED, ABS>(a, b, c);
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+        d[i].x = a[i];
+        a[i] = d[i].y;
+    }
+#pragma unroll
+    for (int q = 0; q < 10; ++q) {
+        g[q].x = b[q];
+        b[q] = g[q].y;
+    }
+    collide_r<float, SCALED, ABS>(a, b, c);
+#pragma unroll
+    for (int i = 0; i < 9; ++i) d[i].y = a[i];
+#pragma unroll
+    for (int q = 0; q < 10; ++q) g[q].y = b[q];
 }
 
 }  // namespace lbmhd

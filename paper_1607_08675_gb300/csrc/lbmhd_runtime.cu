@@ -255,10 +255,13 @@ int lbmhd_create(int nx, int ny, const lbmhd_params* p, lbmhd_t** out) {
     h->d_diag = (double*)mem[3];
     h->d_flag = (int*)mem[4];
     cudaMemsetAsync(h->d_flag, 0, sizeof(int), h->stream);
-    // Default launch shape, measured on GB300: four nodes per thread in
-    // 64-thread blocks for FP32 storage (8192^2 46.0K MLUPS, 1.03x the measured
-    // copy bandwidth), eight nodes (16-byte loads) in 32-thread blocks for FP16
-    // storage (82.0K, 0.92x).  FP64 is bound by the FP64 pipe, and one node per
+    // Default launch shape, measured on GB300: two nodes per thread in
+    // 128-thread blocks for FP32 storage, whose collision then runs two-wide
+    // (us per step, four nodes in 64-thread blocks / this: 256^2 3.2 / 2.9, 512^2
+    // 6.0 / 5.4, 8192 x 64 10.1 / 8.8, 2048^2 98.7 / 95.9, 8192^2 1467 / 1463, the
+    // copy bandwidth).  FP16 storage: eight nodes (16-byte loads) in 32-thread
+    // blocks, 82.0K MLUPS at 8192^2, but four in 64-thread blocks up to 2^20 - 1
+    // nodes (512^2 5.0 / 4.2, 768^2 7.6 / 7.4, 1024^2 12.5 / 12.8).  FP64 is bound by the FP64 pipe, and one node per
     // thread in 64-thread blocks spreads it best at every size (us per step, two
     // nodes in 128-thread blocks / this: 64^2 13.2 / 6.6, 256^2 24.4 / 21.6,
     // 1024^2 303.9 / 295.4).  Double-word FF: two nodes in 256-thread blocks,
@@ -268,7 +271,7 @@ int lbmhd_create(int nx, int ny, const lbmhd_params* p, lbmhd_t** out) {
     const bool ff_small = p->precision == LBMHD_FF && (long long)nx * ny <= 1LL << 18;
     const int want = p->precision == LBMHD_FP64 || ff_small
                          ? 1
-                         : (p->precision == LBMHD_FF ? 2 : (p->precision == LBMHD_FP16_DEV ? 8 : 4));
+                         : (p->precision != LBMHD_FP16_DEV ? 2 : ((long long)nx * ny < 1LL << 20 ? 4 : 8));
     h->vec = 1;
     for (int v = want; v > 1; v >>= 1)
         if (nx % v == 0) {

@@ -15,6 +15,7 @@
 #include "lbmhd_device.cuh"
 #include "lbmhd_f64.cuh"
 #include "lbmhd_internal.h"
+#include "lbmhd_pair.cuh"
 
 namespace lbmhd {
 
@@ -102,24 +103,18 @@ __device__ __forceinline__ void step_body_h(const unsigned short* __restrict__ s
 
 #pragma unroll
     for (int j = 0; j < W; ++j) {
-        float d0[9], g0[10], d1[9], g1[10];
+        float2 d[9], g[10];
 #pragma unroll
         for (int p = 0; p < kPlanes; ++p) {
             const float2 f2 = __half22float2(*reinterpret_cast<const __half2*>(&raw[p][j]));
-            if (p < 9) {
-                d0[p] = f2.x;
-                d1[p] = f2.y;
-            } else {
-                g0[p - 9] = f2.x;
-                g1[p - 9] = f2.y;
-            }
+            if (p < 9) d[p] = f2;
+            else g[p - 9] = f2;
         }
-        collide<float, true>(d0, g0, c);
-        collide<float, true>(d1, g1, c);
+        if constexpr (V == 2) collide_r<float2, true, false>(d, g, c);
+        else collide_pair_each<true, false>(d, g, c);
 #pragma unroll
         for (int p = 0; p < kPlanes; ++p) {
-            const __half2 h = p < 9 ? __floats2half2_rn(d0[p], d1[p])
-                                    : __floats2half2_rn(g0[p - 9], g1[p - 9]);
+            const __half2 h = __float22half2_rn(p < 9 ? d[p] : g[p - 9]);
             raw[p][j] = *reinterpret_cast<const Word*>(&h);
         }
     }
@@ -191,10 +186,10 @@ __device__ __forceinline__ void step_body(const typename Fmt<P>::S* __restrict__
         }
     }
 
+    if constexpr (P == P_FP64) {  // takes and gives the populations themselves
 #pragma unroll
-    for (int k = 0; k < V; ++k) {
-        R d[9], g[10];
-        if constexpr (P == P_FP64) {  // the populations themselves
+        for (int k = 0; k < V; ++k) {
+            R d[9], g[10];
 #pragma unroll
             for (int i = 0; i < 9; ++i) d[i] = raw[i][k];
 #pragma unroll
@@ -204,12 +199,39 @@ __device__ __forceinline__ void step_body(const typename Fmt<P>::S* __restrict__
             for (int i = 0; i < 9; ++i) raw[i][k] = d[i];
 #pragma unroll
             for (int q = 0; q < 10; ++q) raw[9 + q][k] = g[q];
-        } else {
+        }
+    } else if constexpr (P != P_FF && V % 2 == 0) {  // FP32 storage, two nodes at once
+        constexpr bool ABS = P == P_FP32;
+#pragma unroll
+        for (int k = 0; k < V; k += 2) {
+            float2 d[9], g[10];
+#pragma unroll
+            for (int p = 0; p < kPlanes; ++p) {
+                float2 v = make_float2(raw[p][k], raw[p][k + 1]);
+                if (ABS && p < 9) v = add_(v, dup<float2>(-plane_rest<float>(p)));
+                if (p < 9) d[p] = v;
+                else g[p - 9] = v;
+            }
+            if constexpr (V == 2) collide_r<float2, false, ABS>(d, g, c);
+            else collide_pair_each<false, ABS>(d, g, c);
+#pragma unroll
+            for (int p = 0; p < kPlanes; ++p) {
+                float2 v = p < 9 ? d[p] : g[p - 9];
+                if (ABS && p < 9) v = add_(v, dup<float2>(plane_rest<float>(p)));
+                raw[p][k] = v.x;
+                raw[p][k + 1] = v.y;
+            }
+        }
+    } else {
+#pragma unroll
+        for (int k = 0; k < V; ++k) {
+            R d[9], g[10];
 #pragma unroll
             for (int i = 0; i < 9; ++i) d[i] = Fmt<P>::dec(raw[i][k], i, inv_scale);
 #pragma unroll
             for (int q = 0; q < 10; ++q) g[q] = Fmt<P>::dec(raw[9 + q][k], 9 + q, inv_scale);
-            collide<R, Fmt<P>::kScaled>(d, g, c);
+            if constexpr (P == P_FF) collide(d, g, c);
+            else collide_r<float, Fmt<P>::kScaled, P == P_FP32>(d, g, c);
 #pragma unroll
             for (int i = 0; i < 9; ++i) raw[i][k] = Fmt<P>::enc(d[i], i, scale);
 #pragma unroll
@@ -261,7 +283,7 @@ __host__ __device__ inline Coll<R> make_coll_t(double tn, double te, double k18,
 
 // Collision parameters of a storage format: FP16 deviations keep their
 // storage scale through the collision, so the LES constants are divided by
-// it (see collide<R, true>).
+// it (see SCALED in lbmhd_device.cuh).
 template <class R>
 inline Coll<R> coll_for_prec(const HostColl& h, int prec) {
     Coll<R> c = make_coll_t<R>(h.tn, h.te, h.k18, h.k36, h.s5, h.s6, h.s7, h.s8, h.les, h.tie5,

@@ -149,7 +149,7 @@ __global__ void __launch_bounds__(W) step_tma_kernel(const typename Fmt<P>::S* _
                                      blockIdx.x + issued * gridDim.x, tiles_x, nx, ny, ps);
             ++issued;
         }
-        collide<R, Fmt<P>::kScaled>(d, g, c);
+        collide_r<R, Fmt<P>::kScaled, P == P_FP32>(d, g, c);
         S* out = dst + (long long)y * nx + x0 + tid;
 #pragma unroll
         for (int i = 0; i < 9; ++i) out[i * ps] = Fmt<P>::enc(d[i], i, scale);
