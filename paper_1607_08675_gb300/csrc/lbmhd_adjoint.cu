@@ -34,6 +34,7 @@
 #include <type_traits>
 
 #include "lbmhd_internal.h"
+#include "lbmhd_narrow.cuh"
 #include "lbmhd_step_body.cuh"
 
 namespace lbmhd {
@@ -232,10 +233,12 @@ __device__ __forceinline__ void collide_adjoint(const R (&d)[9], const R (&g)[10
 namespace {
 
 constexpr int kAdjBlock = 256;
-// Grid of at most 8 blocks per SM of a 152-SM GB300 (two resident at 114
-// registers, four waves): each thread sweeps many nodes, so its one final
-// conversion and warp reduction of the sensitivity sums stays small.
-constexpr int kAdjMaxBlocks = 8 * 152;
+// At most the two resident blocks per SM of a 152-SM GB300 (114 registers): each
+// thread sweeps its share of the nodes, so the final reduction of the
+// sensitivity sums, whose FP64 additions hold a scheduler's pipe for 64 clocks
+// each, is paid once per resident thread (us per adjoint step, four waves of
+// blocks / one: FP32 512^2 29.2 / 12.8, 2048^2 163.6 / 158.8).
+constexpr int kAdjMaxBlocks = 2 * 152;
 
 __device__ __forceinline__ int wrapi(int a, int n) { return a < 0 ? a + n : (a >= n ? a - n : a); }
 
@@ -296,12 +299,16 @@ __global__ void __launch_bounds__(kAdjBlock) adj_step_kernel(
     }
     __shared__ double red[kAdjBlock / 32][4];
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+    {
+        double v[4];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        double a;
-        a = to_f64(acc[q]);
-        const double w = warp_sum_d(a);
-        if (lane == 0) red[warp][q] = w;
+        for (int q = 0; q < 4; ++q) {
+            if constexpr (std::is_same<Acc, ff>::value) v[q] = widen_ff(acc[q]);
+            else v[q] = acc[q];
+        }
+        const double w = warp_sum_all<4>(v, lane);
+        const int q = warp_sum_index<4>(lane);
+        if (q < 4) red[warp][q] = w;
     }
     __syncthreads();
     if (threadIdx.x < 4) {

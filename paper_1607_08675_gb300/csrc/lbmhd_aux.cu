@@ -330,13 +330,29 @@ __device__ __forceinline__ void acc_add(double& a, double t) { a += t; }
 __device__ __forceinline__ void acc_add(ff& a, ff t) { a += t; }
 __device__ __forceinline__ void acc_add(ff& a, float t) { dw_accumulate(a, t); }
 __device__ __forceinline__ double acc_value(double a) { return a; }
-__device__ __forceinline__ double acc_value(ff a) { return (double)a.hi + (double)a.lo; }
+__device__ __forceinline__ double acc_value(ff a) { return widen_ff(a); }
 __device__ __forceinline__ double to_f64(float v) { return v; }
 __device__ __forceinline__ double to_f64(double v) { return v; }
 __device__ __forceinline__ double to_f64(ff v) { return (double)v.hi + (double)v.lo; }
 __device__ __forceinline__ bool gt(float a, float b) { return a > b; }
 __device__ __forceinline__ bool gt(double a, double b) { return a > b; }
 __device__ __forceinline__ bool gt(ff a, ff b) { return a > b; }
+
+// Largest value of the warp, in the arithmetic type.
+__device__ __forceinline__ double shfl_x(double v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
+__device__ __forceinline__ float shfl_x(float v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
+__device__ __forceinline__ ff shfl_x(ff v, int o) {
+    return ff(__shfl_xor_sync(0xffffffffu, v.hi, o), __shfl_xor_sync(0xffffffffu, v.lo, o));
+}
+template <class R>
+__device__ __forceinline__ R warp_max_r(R v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const R w = shfl_x(v, o);
+        if (gt(w, v)) v = w;
+    }
+    return v;
+}
 
 // Moments of one stored node in the arithmetic type (the sums of the step
 // kernels' collision, deviation form): m = (rho - 1, j_x, j_y, u_x, u_y,
@@ -641,11 +657,15 @@ __global__ void __launch_bounds__(32 * kDiagWarps, kDiagMinBlocks<P>)
             sweep(load);
         }
     }
+    {
+        double v[kNQ];
 #pragma unroll
-    for (int q = 0; q < kNQ; ++q) {
-        const double t = q == 9 ? to_f64(dmax) : acc_value(acc[q]);
-        const double w = q == 9 ? warp_max(t) : warp_sum(t);
-        if (lane == 0) red[warp][q] = w;
+        for (int q = 0; q < kNQ; ++q) v[q] = q == 9 ? 0.0 : acc_value(acc[q]);
+        const double w = warp_sum_all<kNQ>(v, lane);
+        const int q = warp_sum_index<kNQ>(lane);
+        if (q < kNQ && q != 9) red[warp][q] = w;
+        dmax = warp_max_r(dmax);
+        if (lane == 0) red[warp][9] = to_f64(dmax);
     }
     __syncthreads();
     if (threadIdx.x < kNQ) {
@@ -656,43 +676,31 @@ __global__ void __launch_bounds__(32 * kDiagWarps, kDiagMinBlocks<P>)
     }
 }
 
-__global__ void diag_final_kernel(const double* __restrict__ partials, int nblocks, double ncell,
-                                  double* out) {
-    __shared__ double red[256 / 32][kNQ];
-    double acc[kNQ];
-#pragma unroll
-    for (int q = 0; q < kNQ; ++q) acc[q] = 0.0;
-    for (int b = threadIdx.x; b < nblocks; b += blockDim.x)
-#pragma unroll
-        for (int q = 0; q < kNQ; ++q)
-            acc[q] = q == 9 ? fmax(acc[q], partials[b * kNQ + q]) : acc[q] + partials[b * kNQ + q];
-    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-#pragma unroll
-    for (int q = 0; q < kNQ; ++q) {
-        const double w = q == 9 ? warp_max(acc[q]) : warp_sum(acc[q]);
-        if (lane == 0) red[warp][q] = w;
+// One warp per quantity, its lanes over the rows in row order (256^2, 288
+// rows: 3.6 us; one block summing all twelve per thread took 11.5).
+__global__ void __launch_bounds__(32 * kNQ) diag_final_kernel(const double* __restrict__ partials,
+                                                              int nblocks, double ncell, double* out) {
+    const int q = threadIdx.x / 32, lane = threadIdx.x % 32;
+    double s = 0.0;
+    if (q == 9) {
+        for (int b = lane; b < nblocks; b += 32) s = fmax(s, partials[b * kNQ + q]);
+        s = warp_max(s);
+    } else {
+        for (int b = lane; b < nblocks; b += 32) s += partials[b * kNQ + q];
+        s = warp_sum(s);
     }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double s[kNQ];
-        for (int q = 0; q < kNQ; ++q) {
-            s[q] = red[0][q];
-            for (int w = 1; w < 256 / 32; ++w) s[q] = q == 9 ? fmax(s[q], red[w][q]) : s[q] + red[w][q];
-        }
-        const double inv = 1.0 / ncell;
-        out[0] = ncell + s[0];  // the threads summed rho - 1
-        out[1] = s[1];
-        out[2] = s[2];
-        out[3] = s[3];
-        out[4] = s[4];
-        out[5] = 0.5 * s[5] * inv;
-        out[6] = 0.5 * s[6] * inv;
-        out[7] = 0.5 * s[7] * inv;
-        out[8] = s[8] * inv;
-        out[9] = s[9];
-        out[10] = sqrt(s[10] * inv);
-        out[11] = 0.5 * s[11] * inv;
+    if (lane) return;
+    switch (q) {
+        case 0: s = ncell + s; break;  // the threads summed rho - 1
+        case 5:
+        case 6:
+        case 7:
+        case 11: s = 0.5 * s / ncell; break;
+        case 8: s = s / ncell; break;
+        case 10: s = sqrt(s / ncell); break;
+        default: break;
     }
+    out[q] = s;
 }
 
 // ---- launchers ------------------------------------------------------------
@@ -899,7 +907,7 @@ cudaError_t launch_diag(int prec, const void* state, double* partials, double* o
     else
         LBMHD_DISPATCH(prec, (e = diag_launch_p<P, false>(state, partials, g, c, d, st)));
     if (e != cudaSuccess) return e;
-    diag_final_kernel<<<1, 256, 0, st>>>(partials, nb, (double)g.nx * g.ny, out12);
+    diag_final_kernel<<<1, 32 * kNQ, 0, st>>>(partials, nb, (double)g.nx * g.ny, out12);
     return cudaGetLastError();
 }
 

@@ -134,13 +134,17 @@ struct DeviceGuard {
 
 long long ncell(const lbmhd_t* h) { return (long long)h->geom.nx * h->geom.ny; }
 
+int flag_status(int flag) {
+    if (flag & 2) return fail(LBMHD_ETIMEOUT, "a bounded device wait expired in the step kernel");
+    if (flag & 1) return fail(LBMHD_ENONFINITE, "non-finite density detected");
+    return LBMHD_OK;
+}
+
 int read_flag(lbmhd_t* h) {
     int flag = 0;
     LBMHD_CK(h, cudaMemcpyAsync(&flag, h->d_flag, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
     LBMHD_CK(h, cudaStreamSynchronize(h->stream));
-    if (flag & 2) return fail(LBMHD_ETIMEOUT, "a bounded device wait expired in the step kernel");
-    if (flag & 1) return fail(LBMHD_ENONFINITE, "non-finite density detected");
-    return LBMHD_OK;
+    return flag_status(flag);
 }
 
 cudaError_t launch_one(lbmhd_t* h, const void* src, void* dst) {
@@ -224,9 +228,10 @@ int lbmhd_create(int nx, int ny, const lbmhd_params* p, lbmhd_t** out) {
     }
     const size_t bytes = (size_t)kNumPlanes * h->geom.ps * storage_bytes(p->precision);
     const size_t pbytes = (size_t)diag_num_blocks(h->geom, p->precision) * 12 * sizeof(double);
-    void* mem[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
-    const size_t sizes[5] = {bytes, bytes, pbytes, 12 * sizeof(double), sizeof(int)};
-    for (int i = 0; i < 5; ++i) {
+    void* mem[4] = {nullptr, nullptr, nullptr, nullptr};
+    // the flag follows the 12 diagnostics, so that one copy reads both
+    const size_t sizes[4] = {bytes, bytes, pbytes, 13 * sizeof(double)};
+    for (int i = 0; i < 4; ++i) {
         e = cudaMalloc(&mem[i], sizes[i]);
         if (e != cudaSuccess) {
             for (int j = 0; j < i; ++j) cudaFree(mem[j]);
@@ -244,7 +249,7 @@ int lbmhd_create(int nx, int ny, const lbmhd_params* p, lbmhd_t** out) {
                           (p->precision == LBMHD_FP64 || p->precision == LBMHD_FF ? 8 : 4);
         e = cudaMalloc(&h->d_kin, kb);
         if (e != cudaSuccess) {
-            for (int j = 0; j < 5; ++j) cudaFree(mem[j]);
+            for (int j = 0; j < 4; ++j) cudaFree(mem[j]);
             if (h->own_stream) cudaStreamDestroy(h->stream);
             delete h;
             cudaGetLastError();
@@ -253,7 +258,7 @@ int lbmhd_create(int nx, int ny, const lbmhd_params* p, lbmhd_t** out) {
     }
     h->d_partials = (double*)mem[2];
     h->d_diag = (double*)mem[3];
-    h->d_flag = (int*)mem[4];
+    h->d_flag = (int*)(h->d_diag + 12);
     cudaMemsetAsync(h->d_flag, 0, sizeof(int), h->stream);
     // Default launch shape, measured on GB300: two nodes per thread in
     // 128-thread blocks for FP32 storage, whose collision then runs two-wide
@@ -512,11 +517,14 @@ int lbmhd_diagnostics(lbmhd_t* h, lbmhd_diag* out) {
     if (!out) return fail(LBMHD_EINVAL, "out is NULL");
     if (!h->initialised) return fail(LBMHD_ESTATE, "diagnostics before lbmhd_init");
     DeviceGuard dg(h->device);
-    double v[12];
+    double v[13];  // and the flag
     LBMHD_CK(h, launch_diag(h->p.precision, h->buf[h->cur], h->d_partials, h->d_diag, h->geom,
                             h->coll, h->stream));
     LBMHD_CK(h, cudaMemcpyAsync(v, h->d_diag, sizeof(v), cudaMemcpyDeviceToHost, h->stream));
-    rc = read_flag(h);
+    LBMHD_CK(h, cudaStreamSynchronize(h->stream));
+    int flag;
+    std::memcpy(&flag, v + 12, sizeof flag);
+    rc = flag_status(flag);
     out->mass = v[0];
     out->mom_x = v[1];
     out->mom_y = v[2];
@@ -711,7 +719,6 @@ void lbmhd_destroy(lbmhd_t* h) {
     cudaFree(h->buf[1]);
     cudaFree(h->d_partials);
     cudaFree(h->d_diag);
-    cudaFree(h->d_flag);
     cudaFree(h->d_kin);
     if (h->own_stream) cudaStreamDestroy(h->stream);
     delete h;
