@@ -127,9 +127,13 @@ struct lbmhd_batch_t {
     int* d_unit_run;
     void* d_mom;  // les 2, 3: every run's five moment planes
     unsigned nunits;
+    int pipe;           // kPipeSteps steps per pass where that many follow each other
+    bool peven;         // every nx is even
+    unsigned pnunits;
+    int* d_punit_run;
     unsigned* d_bar;
     int* d_flag;
-    int vec, block, spl, grid;
+    int vec, block, spl, grid, sms;
     int cur;
     int64_t steps, launches;
     std::vector<char> run_init;
@@ -232,8 +236,11 @@ int kin_seglen(int ny) {
 template <class R>
 int upload_runs_t(lbmhd_batch_t* b) {
     std::vector<RunDev<R>> rd(b->nruns);
-    std::vector<int> map;
+    std::vector<int> map, pmap, pstrips(b->nruns);
     unsigned unit = 0;
+    const int pseglen =
+        b->pipe ? batch_pipe_plan(b->p.precision, b->nruns, b->nx.data(), b->ny.data(), b->sms, pstrips.data()) : 1;
+    b->peven = true;
     long long moff = 0;
     const bool kin = b->p.les >= 2;
     const int ksw = kinetic_fused_strip(b->p.precision);
@@ -252,6 +259,11 @@ int upload_runs_t(lbmhd_batch_t* b) {
         rd[r].kstrips = (b->nx[r] + ksw - 1) / ksw;
         rd[r].kseglen = kin_seglen(b->ny[r]);
         rd[r].c = coll_for_prec<R>(hc, b->p.precision);
+        rd[r].punit0 = (unsigned)pmap.size();
+        rd[r].pstrips = pstrips[r];
+        rd[r].pseglen = pseglen;
+        b->peven = b->peven && b->nx[r] % 2 == 0;
+        if (b->pipe) pmap.insert(pmap.end(), (size_t)pstrips[r] * ((b->ny[r] + pseglen - 1) / pseglen), r);
         const unsigned units =
             kin && b->vec == 1
                 ? (unsigned)rd[r].kstrips * (unsigned)((b->ny[r] + rd[r].kseglen - 1) / rd[r].kseglen)
@@ -262,8 +274,16 @@ int upload_runs_t(lbmhd_batch_t* b) {
     b->nunits = unit;
     if (b->d_runs) cudaFree(b->d_runs);
     if (b->d_unit_run) cudaFree(b->d_unit_run);
+    if (b->d_punit_run) cudaFree(b->d_punit_run);
     b->d_runs = nullptr;
     b->d_unit_run = nullptr;
+    b->d_punit_run = nullptr;
+    b->pnunits = (unsigned)pmap.size();
+    if (b->pnunits) {
+        LBMHD_BCK(b, cudaMalloc((void**)&b->d_punit_run, pmap.size() * sizeof(int)));
+        LBMHD_BCK(b, cudaMemcpy(b->d_punit_run, pmap.data(), pmap.size() * sizeof(int),
+                                cudaMemcpyHostToDevice));
+    }
     LBMHD_BCK(b, cudaMalloc(&b->d_runs, rd.size() * sizeof(RunDev<R>)));
     LBMHD_BCK(b, cudaMalloc((void**)&b->d_unit_run, map.size() * sizeof(int)));
     LBMHD_BCK(b, cudaMemcpy(b->d_runs, rd.data(), rd.size() * sizeof(RunDev<R>),
@@ -273,8 +293,16 @@ int upload_runs_t(lbmhd_batch_t* b) {
     return LBMHD_OK;
 }
 
-// (Re)build the unit map and the co-resident grid for the current shape.
+// The ensemble takes several steps per pass where a lattice of its size would.
+bool batch_pipe_ok(const lbmhd_batch_t* b) {
+    long long nodes = 0;
+    for (int r = 0; r < b->nruns; ++r) nodes += (long long)b->nx[r] * b->ny[r];
+    return b->p.les < 2 && pipe_ok(b->p.precision, nodes);
+}
+
+// (Re)build the unit maps and the co-resident grid for the current shape.
 int configure(lbmhd_batch_t* b) {
+    LBMHD_BCK(b, cudaDeviceGetAttribute(&b->sms, cudaDevAttrMultiProcessorCount, b->device));
     int rc = b->p.precision == LBMHD_FP64 ? upload_runs_t<double>(b)
              : b->p.precision == LBMHD_FF ? upload_runs_t<ff>(b)
                                           : upload_runs_t<float>(b);
@@ -287,11 +315,10 @@ int configure(lbmhd_batch_t* b) {
     }
     const void* k = pick_kernel(b->p.precision, b->vec);
     if (!k) return bfail(LBMHD_EINVAL, "no batched kernel for this precision / vector width");
-    int per_sm = 0, sms = 0;
+    int per_sm = 0;
     LBMHD_BCK(b, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, b->block, 0));
-    LBMHD_BCK(b, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, b->device));
     if (per_sm < 1) return bfail(LBMHD_EINVAL, "batched kernel cannot be resident at this shape");
-    long long grid = (long long)per_sm * sms;
+    long long grid = (long long)per_sm * b->sms;
     if (grid > (long long)b->nunits) grid = b->nunits;
     b->grid = (int)std::max<long long>(1, grid);
     if (b->graph) cudaGraphExecDestroy(b->graph);
@@ -340,6 +367,14 @@ cudaError_t launch_batch(lbmhd_batch_t* b, int nsteps, int parity) {
     return cudaLaunchKernelExC(&cfg, k, args);
 }
 
+// One pass of kPipeSteps steps over every run.  Not while a barrier arrival is
+// to be dropped (there is no barrier in it).
+bool use_pipe(const lbmhd_batch_t* b) { return b->pipe && b->pnunits && !b->drop_arrival; }
+cudaError_t launch_pass(lbmhd_batch_t* b, int parity) {
+    return launch_batch_pipe(b->p.precision, b->peven, b->d_runs, b->d_punit_run, b->pnunits,
+                             b->buf[parity & 1], b->buf[1 - (parity & 1)], b->stream);
+}
+
 // Capture kGraphLaunches persistent launches (spl steps each) starting at
 // the current buffer parity.  False (with the error cleared) when the
 // driver refuses to capture them.
@@ -352,8 +387,8 @@ bool capture_graph(lbmhd_batch_t* b) {
     int parity = b->cur;
     bool ok = true;
     for (int l = 0; l < kGraphLaunches && ok; ++l) {
-        ok = launch_batch(b, b->spl, parity) == cudaSuccess;
-        parity = (parity + b->spl) & 1;
+        ok = (use_pipe(b) ? launch_pass(b, parity) : launch_batch(b, b->spl, parity)) == cudaSuccess;
+        parity = (parity + (use_pipe(b) ? 1 : b->spl)) & 1;
     }
     const cudaError_t ee = cudaStreamEndCapture(b->stream, &g);
     ok = ok && ee == cudaSuccess && g;
@@ -365,7 +400,7 @@ bool capture_graph(lbmhd_batch_t* b) {
         return false;
     }
     b->graph_cur = b->cur;
-    b->graph_len = b->spl * kGraphLaunches;
+    b->graph_len = (use_pipe(b) ? kPipeSteps : b->spl) * kGraphLaunches;
     return true;
 }
 
@@ -576,6 +611,7 @@ int lbmhd_batch_create(int nruns, const int* nx, const int* ny, const double* ta
         b->block = 128;
         b->spl = 1;
     }
+    b->pipe = batch_pipe_ok(b);
     int rc = configure(b);
     if (rc) {
         lbmhd_batch_destroy(b);
@@ -585,7 +621,7 @@ int lbmhd_batch_create(int nruns, const int* nx, const int* ny, const double* ta
     return LBMHD_OK;
 }
 
-int lbmhd_batch_set_launch(lbmhd_batch_t* b, int vec, int block, int steps_per_launch) {
+static int set_shape(lbmhd_batch_t* b, int vec, int block, int steps_per_launch) {
     int rc = check_batch(b);
     if (rc) return rc;
     if (b->p.les >= 2) {
@@ -607,6 +643,14 @@ int lbmhd_batch_set_launch(lbmhd_batch_t* b, int vec, int block, int steps_per_l
     b->block = block;
     b->spl = steps_per_launch;
     return configure(b);
+}
+
+int lbmhd_batch_set_launch(lbmhd_batch_t* b, int vec, int block, int steps_per_launch) {
+    const int was = b ? b->pipe : 0;
+    if (b) b->pipe = 0;  // the shape that was asked for
+    const int rc = set_shape(b, vec, block, steps_per_launch);
+    if (rc && b) b->pipe = was;
+    return rc;
 }
 
 int lbmhd_batch_get_launch(const lbmhd_batch_t* b, int* vec, int* block, int* steps_per_launch) {
@@ -651,10 +695,13 @@ int lbmhd_batch_step(lbmhd_batch_t* b, int n) {
     for (int r = 0; r < b->nruns; ++r)
         if (!b->run_init[r]) return bfail(LBMHD_ESTATE, "every run must be initialised first");
     int done = 0;
-    const int chunk = b->spl * kGraphLaunches;
+    const bool pipe = use_pipe(b);
+    const int per = pipe ? kPipeSteps : b->spl;  // steps of a launch, and buffer swaps
+    const int swaps = pipe ? 1 : b->spl;
+    const int chunk = per * kGraphLaunches;
     while (done < n) {
         if (n - done >= chunk && b->capturable && !b->drop_arrival) {
-            if (!b->graph || b->graph_cur != b->cur) {
+            if (!b->graph || b->graph_cur != b->cur || b->graph_len != chunk) {
                 if (b->graph) cudaGraphExecDestroy(b->graph);
                 b->graph = nullptr;
                 if (!capture_graph(b)) {
@@ -665,10 +712,18 @@ int lbmhd_batch_step(lbmhd_batch_t* b, int n) {
                 }
             }
             LBMHD_BCK(b, cudaGraphLaunch(b->graph, b->stream));
-            b->cur = (b->cur + chunk) & 1;
+            b->cur = (b->cur + swaps * kGraphLaunches) & 1;
             b->launches += kGraphLaunches;
             b->steps += chunk;
             done += chunk;
+            continue;
+        }
+        if (pipe && n - done >= kPipeSteps) {
+            LBMHD_BCK(b, launch_pass(b, b->cur));
+            b->cur ^= 1;
+            ++b->launches;
+            b->steps += kPipeSteps;
+            done += kPipeSteps;
             continue;
         }
         const int k = std::min(b->spl, n - done);
@@ -746,6 +801,9 @@ int lbmhd_batch_autotune(lbmhd_batch_t* b, const char* cache_path, int trial_ste
     if (trial_steps < 2) return bfail(LBMHD_EINVAL, "trial_steps must be >= 2");
     for (int r = 0; r < b->nruns; ++r)
         if (b->run_init[r]) return bfail(LBMHD_ESTATE, "autotune runs before lbmhd_batch_init");
+    // the shapes are those of the one-step kernel; ensembles that take several
+    // steps per pass do so whatever was set before
+    b->pipe = batch_pipe_ok(b);
     const std::string key = tune_key(b);
     std::lock_guard<std::mutex> lock(g_tune_mu);
     std::map<std::string, std::vector<double>> cache;
@@ -753,7 +811,7 @@ int lbmhd_batch_autotune(lbmhd_batch_t* b, const char* cache_path, int trial_ste
         cache = load_cache(cache_path);
         auto it = cache.find(key);
         if (it != cache.end()) {
-            rc = lbmhd_batch_set_launch(b, (int)it->second[0], (int)it->second[1],
+            rc = set_shape(b, (int)it->second[0], (int)it->second[1],
                                         (int)it->second[2]);
             if (rc == LBMHD_OK) {
                 if (best_mlups) *best_mlups = it->second[3];
@@ -792,7 +850,7 @@ int lbmhd_batch_autotune(lbmhd_batch_t* b, const char* cache_path, int trial_ste
     for (int v : vecs)
         for (int bl : blocks)
             for (int s : spls) {
-                if (lbmhd_batch_set_launch(b, v, bl, s) != LBMHD_OK) continue;
+                if (set_shape(b, v, bl, s) != LBMHD_OK) continue;
                 const int warm = std::min(s, trial_steps);
                 LBMHD_BCK(b, launch_batch(b, warm, b->cur));
                 b->cur = (b->cur + warm) & 1;
@@ -816,11 +874,26 @@ int lbmhd_batch_autotune(lbmhd_batch_t* b, const char* cache_path, int trial_ste
                     bs = s;
                 }
             }
+    if (use_pipe(b)) {
+        LBMHD_BCK(b, launch_pass(b, b->cur));
+        b->cur ^= 1;
+        LBMHD_BCK(b, cudaEventRecord(e0, b->stream));
+        const int passes = std::max(1, trial_steps / kPipeSteps);
+        for (int l = 0; l < passes; ++l) {
+            LBMHD_BCK(b, launch_pass(b, b->cur));
+            b->cur ^= 1;
+        }
+        LBMHD_BCK(b, cudaEventRecord(e1, b->stream));
+        LBMHD_BCK(b, cudaEventSynchronize(e1));
+        float ms = 0.f;
+        LBMHD_BCK(b, cudaEventElapsedTime(&ms, e0, e1));
+        best = std::max(best, (double)cells * passes * kPipeSteps / (ms * 1e-3) / 1e6);
+    }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     rc = read_batch_flag(b);
     if (rc) return rc;
-    rc = lbmhd_batch_set_launch(b, bv, bb, bs);
+    rc = set_shape(b, bv, bb, bs);
     if (rc) return rc;
     if (best_mlups) *best_mlups = best;
     if (cache_path && *cache_path) {
@@ -839,6 +912,7 @@ void lbmhd_batch_destroy(lbmhd_batch_t* b) {
     cudaFree(b->buf[1]);
     cudaFree(b->d_runs);
     cudaFree(b->d_unit_run);
+    cudaFree(b->d_punit_run);
     cudaFree(b->d_mom);
     cudaFree(b->d_bar);
     cudaFree(b->d_flag);

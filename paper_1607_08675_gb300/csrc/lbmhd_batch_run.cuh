@@ -16,6 +16,9 @@ struct RunDev {
     unsigned unit0;  // first work unit of the run
     int kstrips;     // fused kinetic kernel: column strips of the run
     int kseglen;     // ... and rows per segment (units = strips x segments)
+    unsigned punit0;  // several steps per pass: first unit of the run,
+    int pstrips;      // its column strips
+    int pseglen;      // and rows per segment
     Coll<R> c;
 };
 

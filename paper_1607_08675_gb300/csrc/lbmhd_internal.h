@@ -59,9 +59,16 @@ bool step_variant_ok(int prec, int vec, int nx);
 // (lbmhd_step_pipe.cu): the bits of as many launch_step calls.  pipe_ok: the
 // storage format has the kernel and the lattice is large enough for it.
 constexpr int kPipeSteps = 4;
-bool pipe_ok(int prec, const Geom& g);
+bool pipe_ok(int prec, long long nodes);
 cudaError_t launch_pipe(int prec, int steps, const void* src, void* dst, const Geom& g,
                         const HostColl& c, int sm_count, cudaStream_t st);
+
+// kPipeSteps steps of every run of an ensemble in one pass.  batch_pipe_plan
+// gives the rows of a segment and each run's strips (RunDev::pseglen,
+// pstrips, units = strips x segments); even: every run's nx is even.
+int batch_pipe_plan(int prec, int nruns, const int* nx, const int* ny, int sm_count, int* strips);
+cudaError_t launch_batch_pipe(int prec, bool even, const void* runs, const int* unit_run,
+                              unsigned nunits, const void* src, void* dst, cudaStream_t st);
 
 // TMA-staged step (lbmhd_step_tma.cu): W threads = nodes per row tile,
 // persistent grid of `grid` CTAs; a timed-out wait sets bit 2 of *status.

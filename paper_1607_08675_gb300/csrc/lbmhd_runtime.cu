@@ -287,7 +287,7 @@ int lbmhd_create(int nx, int ny, const lbmhd_params* p, lbmhd_t** out) {
                : h->vec == 4 || p->precision == LBMHD_FP64 ? 64
                : p->precision == LBMHD_FF && !ff_small ? 256 : 128;
     h->tma_w = 0;
-    h->pipe = h->coll.kin == 0 && pipe_ok(p->precision, h->geom);
+    h->pipe = h->coll.kin == 0 && pipe_ok(p->precision, (long long)nx * ny);
     // Kinetic steps: the fused kernel where it is faster (measured at 8192^2
     // / 4096^2, MLUPS fused vs two-pass: FP32 les 2 33.5K vs 23.7K, les 3
     // 37.1K vs 22.3K; FP16 38.9K vs 26.6K; FF les 3 8.2K vs 7.2K), the

@@ -39,6 +39,9 @@
 // c_y = 0 planes -- L1 takes what shared memory leaves, and it holds the
 // rows in flight; with the largest shared-memory carve-out S = 2 fell to
 // 57 G, and any spilled register costs half the rate.
+#include <algorithm>
+
+#include "lbmhd_batch_run.cuh"
 #include "lbmhd_cp_async.cuh"
 #include "lbmhd_internal.h"
 #include "lbmhd_pair.cuh"
@@ -133,21 +136,30 @@ __host__ __device__ constexpr int pipe_warps(int prec, int steps) {
     return prec == P_FP16_DEV || steps == 2 ? 4 : (steps == 3 ? 3 : 2);
 }
 
-// AL: nx is even, so a lane's pair is one aligned word in every row.
+// The shared memory of one warp.
 template <int P, int S, bool AL>
-__global__ void __launch_bounds__(32, 4 * pipe_warps(P, S))
-    pipe_kernel(const typename Fmt<P>::S* __restrict__ src, typename Fmt<P>::S* __restrict__ dst,
-                int nx, int ny, long long ps, int strips, int seglen, Coll<float> c) {
+struct PipeShared {
+    using Q = typename PairOf<P>::T;
+    // cp.async moves 4 or 8 bytes: odd rows of FP16 are loaded directly
+    static constexpr bool PF = AL || P != P_FP16_DEV;
+    Q pre[PF ? kPlanes : 1][32];  // the fetched row
+    Q keep[S - 1][9][32];         // each step's last row, c_y = 0
+};
+
+// One warp: S steps of rows [y0, y1) of one strip of a lattice.  AL: nx is
+// even, so a lane's pair is one aligned word in every row.
+template <int P, int S, bool AL>
+__device__ __forceinline__ void pipe_body(const typename Fmt<P>::S* __restrict__ src,
+                                          typename Fmt<P>::S* __restrict__ dst, int nx, int ny,
+                                          long long ps, int strip, int y0, int y1,
+                                          const Coll<float>& c, PipeShared<P, S, AL>& sh) {
     using T = typename Fmt<P>::S;
     using Q = typename PairOf<P>::T;
     constexpr int HL = PipeShape<S>::kHalo, U = PipeShape<S>::kUseful;
-    // cp.async moves 4 or 8 bytes: odd rows of FP16 are loaded directly
-    constexpr bool PF = AL || P != P_FP16_DEV;
-    __shared__ Q pre[PF ? kPlanes : 1][32];  // the fetched row
-    __shared__ Q keep[S - 1][9][32];         // each step's last row, c_y = 0
+    constexpr bool PF = PipeShared<P, S, AL>::PF;
+    auto& pre = sh.pre;
+    auto& keep = sh.keep;
     const int lane = threadIdx.x;
-    const int strip = (int)(blockIdx.x % (unsigned)strips), seg = (int)(blockIdx.x / (unsigned)strips);
-    const int y0 = seg * seglen, y1 = min(y0 + seglen, ny);
     const int x = strip * U - HL + 2 * lane;  // this lane's first column, unwrapped
     int xa = x % nx;
     if (xa < 0) xa += nx;
@@ -261,6 +273,34 @@ __global__ void __launch_bounds__(32, 4 * pipe_warps(P, S))
     }
 }
 
+template <int P, int S, bool AL>
+__global__ void __launch_bounds__(32, 4 * pipe_warps(P, S))
+    pipe_kernel(const typename Fmt<P>::S* __restrict__ src, typename Fmt<P>::S* __restrict__ dst,
+                int nx, int ny, long long ps, int strips, int seglen, Coll<float> c) {
+    __shared__ PipeShared<P, S, AL> sh;
+    const int strip = (int)(blockIdx.x % (unsigned)strips), seg = (int)(blockIdx.x / (unsigned)strips);
+    const int y0 = seg * seglen;
+    pipe_body<P, S, AL>(src, dst, nx, ny, ps, strip, y0, min(y0 + seglen, ny), c, sh);
+}
+
+// kPipeSteps steps of every run of an ensemble, a warp per strip-segment of a
+// run, so every run gets the bits of its own lattice.  The run's rates are
+// read by every lane into registers, so FP16 has the registers of three
+// warps per scheduler here, not four.
+constexpr int batch_pipe_warps(int prec) { return prec == P_FP16_DEV ? 3 : 2; }
+template <int P, bool AL>
+__global__ void __launch_bounds__(32, 4 * batch_pipe_warps(P))
+    batch_pipe_kernel(const RunDev<float>* __restrict__ runs, const int* __restrict__ unit_run,
+                      const typename Fmt<P>::S* __restrict__ src, typename Fmt<P>::S* __restrict__ dst) {
+    __shared__ PipeShared<P, kPipeSteps, AL> sh;
+    const RunDev<float>& rd = runs[unit_run[blockIdx.x]];
+    const int l = (int)(blockIdx.x - rd.punit0);
+    const int strip = l % rd.pstrips, y0 = l / rd.pstrips * rd.pseglen;
+    const Coll<float> c = rd.c;
+    pipe_body<P, kPipeSteps, AL>(src + rd.off, dst + rd.off, rd.nx, rd.ny, rd.ps, strip, y0,
+                                 min(y0 + rd.pseglen, rd.ny), c, sh);
+}
+
 // Rows per segment, at most 96 (longer ones let neighbouring strips drift
 // apart and their shared columns leave L2: 8192^2, S = 4, 96 rows 127.9 G,
 // 192 rows 124 G).  The time of a launch is its rounds of resident warps
@@ -270,18 +310,17 @@ __global__ void __launch_bounds__(32, 4 * pipe_warps(P, S))
 // 1.25 at one warp, 2.05 at two; S = 3 2.39 at three).  Within 3% of the best
 // length of a sweep at 1024^2, 1999 x 1201, 2048^2 and 8192^2, where a length
 // that leaves part of a round empty costs up to 60%.
-template <int P, int S>
-int pipe_seglen(int strips, int ny, int sm_count) {
-    constexpr int kMost = 96;
-    constexpr double a = S == 2 ? 0.8 : (S == 3 ? 0.56 : 0.45), b = S == 2 ? 0.6 : (S == 3 ? 0.61 : 0.8);
+template <class Units>
+int best_seglen(int S, int warps, int most, int sm_count, Units units_of) {
+    const double a = S == 2 ? 0.8 : (S == 3 ? 0.56 : 0.45), b = S == 2 ? 0.6 : (S == 3 ? 0.61 : 0.8);
     const double sched = 4.0 * sm_count;
-    const long long resident = 4LL * pipe_warps(P, S) * sm_count;
+    const long long resident = 4LL * warps * sm_count;
     int best = 1;
     double best_t = 1e300;
-    for (int len = 1; len <= kMost && len <= ny; ++len) {
-        const long long units = (long long)strips * ((ny + len - 1) / len);
+    for (int len = 1; len <= std::min(most, 96); ++len) {
+        const long long units = units_of(len);
         const long long rounds = units / resident, rest = units % resident;
-        double t = (double)rounds * (a + b * pipe_warps(P, S));
+        double t = (double)rounds * (a + b * warps);
         if (rest) t += a + b * (rest > sched ? (double)rest / sched : 1.0);
         t *= len + 2 * (S - 1) + 1;
         if (t < best_t) {
@@ -297,7 +336,9 @@ cudaError_t launch_pipe_t(const void* src, void* dst, const Geom& g, const HostC
                           cudaStream_t st) {
     using T = typename Fmt<P>::S;
     const int strips = (g.nx + PipeShape<S>::kUseful - 1) / PipeShape<S>::kUseful;
-    const int seglen = pipe_seglen<P, S>(strips, g.ny, sm_count);
+    const int seglen = best_seglen(S, pipe_warps(P, S), g.ny, sm_count, [&](int len) {
+        return (long long)strips * ((g.ny + len - 1) / len);
+    });
     const int nseg = (g.ny + seglen - 1) / seglen;
     pipe_kernel<P, S, AL><<<(unsigned)strips * (unsigned)nseg, 32, 0, st>>>(
         (const T*)src, (T*)dst, g.nx, g.ny, g.ps, strips, seglen, coll_for_prec<float>(hc, P));
@@ -318,10 +359,41 @@ cudaError_t launch_pipe_p(int steps, const void* src, void* dst, const Geom& g, 
 
 }  // namespace
 
-bool pipe_ok(int prec, const Geom& g) {
+bool pipe_ok(int prec, long long nodes) {
     if (prec != P_FP32 && prec != P_FP32_DEV && prec != P_FP16_DEV) return false;
-    const long long n = (long long)g.nx * g.ny;
-    return n <= kPipeSmall || 2 * kPlanes * (long long)storage_bytes(prec) * n >= kPipeBytes;
+    return nodes <= kPipeSmall || 2 * kPlanes * (long long)storage_bytes(prec) * nodes >= kPipeBytes;
+}
+
+int batch_pipe_plan(int prec, int nruns, const int* nx, const int* ny, int sm_count, int* strips) {
+    constexpr int U = PipeShape<kPipeSteps>::kUseful;
+    int most = 1;
+    for (int r = 0; r < nruns; ++r) {
+        strips[r] = (nx[r] + U - 1) / U;
+        most = std::max(most, ny[r]);
+    }
+    return best_seglen(kPipeSteps, batch_pipe_warps(prec), most, sm_count, [&](int len) {
+        long long u = 0;
+        for (int r = 0; r < nruns; ++r) u += (long long)strips[r] * ((ny[r] + len - 1) / len);
+        return u;
+    });
+}
+
+cudaError_t launch_batch_pipe(int prec, bool even, const void* runs, const int* unit_run,
+                              unsigned nunits, const void* src, void* dst, cudaStream_t st) {
+    const RunDev<float>* rd = (const RunDev<float>*)runs;
+#define LBMHD_BP(P)                                                                           \
+    case P:                                                                                   \
+        (even ? batch_pipe_kernel<P, true> : batch_pipe_kernel<P, false>)<<<nunits, 32, 0, st>>>( \
+            rd, unit_run, (const Fmt<P>::S*)src, (Fmt<P>::S*)dst);                            \
+        break;
+    switch (prec) {
+        LBMHD_BP(P_FP32)
+        LBMHD_BP(P_FP32_DEV)
+        LBMHD_BP(P_FP16_DEV)
+        default: return cudaErrorInvalidValue;
+    }
+#undef LBMHD_BP
+    return cudaGetLastError();
 }
 
 cudaError_t launch_pipe(int prec, int steps, const void* src, void* dst, const Geom& g,

@@ -86,3 +86,37 @@ def test_finiteness_check_between_launches(L):
     finally:
         L.lbmhd_destroy(h)
     assert np.array_equal(got, raw(L, shape, fields, "fp32", 1, (10,), True)[0])
+
+
+@pytest.mark.parametrize("prec", ["fp32", "fp32_dev", "fp16_dev"])
+@pytest.mark.parametrize("sizes", [[(64, 40), (57, 3), (8, 8)], [(112, 9), (56, 33), (2, 1), (130, 64)],
+                                   [(640, 701), (96, 100), (513, 300)]])
+def test_ensemble_passes_equal_single_lattices(L, prec, sizes):
+    """Runs of uneven sizes, odd and even, one below and one above the size
+    from which an ensemble leaves L2; calls that mix passes of four steps,
+    graph replay and single steps."""
+    nx, ny = [s[0] for s in sizes], [s[1] for s in sizes]
+    tau, cs = [0.55 + 0.02 * i for i in range(len(sizes))], [0.1 + 0.01 * i for i in range(len(sizes))]
+    rates = dict(s5=1.2, s6=1.2, s7=1.3, s8=1.3)
+    calls = (3, 4, 33, 6)
+    f = [inputs.orszag_tang(*s, seed=i, amp=1e-3) for i, s in enumerate(sizes)]
+    b = L.lbmhd_batch_create(nx, ny, tau, tau, cs, L.lbmhd_params_default(precision=prec, **rates))
+    try:
+        for r in range(len(sizes)):
+            L.lbmhd_batch_init(b, r, *f[r])
+        for n in calls:
+            L.lbmhd_batch_step(b, n)
+        assert L.lbmhd_batch_step_count(b) == sum(calls)
+        got = [L.lbmhd_batch_get_state(b, r) for r in range(len(sizes))]
+    finally:
+        L.lbmhd_batch_destroy(b)
+    for r, s in enumerate(sizes):
+        h = L.lbmhd_create(*s, L.lbmhd_params_default(precision=prec, tau_nu=tau[r], tau_eta=tau[r],
+                                                      C_S=cs[r], **rates))
+        try:
+            L.lbmhd_set_launch(h, 1, 64)
+            L.lbmhd_init(h, *f[r])
+            L.lbmhd_step(h, sum(calls))
+            assert np.array_equal(L.lbmhd_get_state(h), got[r]), s
+        finally:
+            L.lbmhd_destroy(h)
