@@ -151,9 +151,10 @@ int lbmhd_init_device(lbmhd_t* h, const double* rho, const double* ux, const dou
                       const double* bx, const double* by);
 
 /* Advance n >= 0 time steps of fused pull-stream and collide (Sec. 1.2 and
- * Sec. 3) over the whole lattice, one per launch; FP32 and FP16 storage with
- * les 0 or 1 advance up to four per launch where steps follow each other
- * (the same bits; not after lbmhd_set_launch).  Asynchronous on the handle's
+ * Sec. 3) over the whole lattice, one per launch; FP32 and FP16 storage
+ * advance up to four (les 0, 1) or two (les 2, 3) per launch where steps
+ * follow each other and the lattice is of a size that gains by it (the same
+ * bits; not after lbmhd_set_launch).  Asynchronous on the handle's
  * stream; long runs replay a captured CUDA graph.  Returns
  * ESTATE before init.  A pending non-finite report (check_finite_every)
  * is returned by the next synchronising call. */

@@ -22,12 +22,13 @@ SOURCES = ["lbmhd_step.cu", "lbmhd_step_pipe.cu", "lbmhd_step_tma.cu", "lbmhd_au
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2",
          "--expt-relaxed-constexpr", "-I", INCLUDE]
-# Per-file flags.  The kinetic-LES kernels and the 3D step are compiled
-# without FMA contraction: kernels of different shape (fused and two-pass;
-# one or two nodes per thread) perform the same operations in the same order
-# but in differently shaped code, and only with every fusion written out is
-# "same operations" also "same bits".
-FILE_FLAGS = {"lbmhd_kinetic.cu": ["-fmad=false"], "lbmhd3.cu": ["-fmad=false"]}
+# Per-file flags.  The kinetic-LES kernels, the passes of several steps and the
+# 3D step are compiled without FMA contraction: kernels of different shape
+# (fused and two-pass; one or several steps; one or two nodes per thread)
+# perform the same operations in the same order but in differently shaped
+# code, and only with every fusion written out is "same operations" also
+# "same bits".
+FILE_FLAGS = {"lbmhd_step_pipe.cu": ["-fmad=false"], "lbmhd_kinetic.cu": ["-fmad=false"], "lbmhd3.cu": ["-fmad=false"]}
 
 
 def nvcc() -> str:

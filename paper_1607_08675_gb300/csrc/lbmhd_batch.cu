@@ -297,7 +297,7 @@ int upload_runs_t(lbmhd_batch_t* b) {
 bool batch_pipe_ok(const lbmhd_batch_t* b) {
     long long nodes = 0;
     for (int r = 0; r < b->nruns; ++r) nodes += (long long)b->nx[r] * b->ny[r];
-    return b->p.les < 2 && pipe_ok(b->p.precision, nodes);
+    return b->p.les < 2 && pipe_steps(b->p.precision, nodes, false) > 0;
 }
 
 // (Re)build the unit maps and the co-resident grid for the current shape.

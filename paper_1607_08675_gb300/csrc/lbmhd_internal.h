@@ -56,12 +56,20 @@ cudaError_t launch_step(int prec, int vec, int block, int max_blocks, const void
 bool step_variant_ok(int prec, int vec, int nx);
 
 // `steps` (2 .. kPipeSteps) time steps in one pass, src -> dst
-// (lbmhd_step_pipe.cu): the bits of as many launch_step calls.  pipe_ok: the
-// storage format has the kernel and the lattice is large enough for it.
+// (lbmhd_step_pipe.cu): the bits of as many launch_step calls.  pipe_steps:
+// the most steps of a pass for a lattice or an ensemble of this many nodes
+// (kin: with a kinetic closure), 0 where single steps are as fast or the
+// format has no such kernel.
 constexpr int kPipeSteps = 4;
-bool pipe_ok(int prec, long long nodes);
+int pipe_steps(int prec, long long nodes, bool kin);
 cudaError_t launch_pipe(int prec, int steps, const void* src, void* dst, const Geom& g,
                         const HostColl& c, int sm_count, cudaStream_t st);
+
+// Two steps of a kinetic closure (g.kin 2 or 3) in one pass, for the same
+// formats: the bits of two launch_step_kinetic calls.
+constexpr int kKinPipeSteps = 2;
+cudaError_t launch_kin_pipe(int prec, const void* src, void* dst, const Geom& g, const HostColl& c,
+                            int sm_count, cudaStream_t st);
 
 // kPipeSteps steps of every run of an ensemble in one pass.  batch_pipe_plan
 // gives the rows of a segment and each run's strips (RunDev::pseglen,
@@ -159,7 +167,7 @@ struct lbmhd_t {
     int* d_flag;
     int vec, block;   // register kernel: nodes per thread, threads per block
     int tma_w;        // > 0: TMA-staged kernel with this tile width
-    int pipe;         // several steps per pass (lbmhd_step_pipe.cu) where steps follow each other
+    int pipe;         // most steps of a pass (lbmhd_step_pipe.cu) where steps follow each other, 0: one per launch
     int kin_two_pass; // les 2, 3: moments pass + step instead of the fused kernel
     int sm_count;
     cudaGraphExec_t graph;

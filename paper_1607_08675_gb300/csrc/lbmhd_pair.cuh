@@ -31,7 +31,10 @@ __device__ __forceinline__ float fma_(float a, float b, float c) { return __fmaf
 __device__ __forceinline__ float neg_(float a) { return -a; }
 __device__ __forceinline__ float abs_(float a) { return fabsf(a); }
 __device__ __forceinline__ float2 add_(float2 a, float2 b) { return __fadd2_rn(a, b); }
-__device__ __forceinline__ float2 mul_(float2 a, float2 b) { return __fmul2_rn(a, b); }
+// A product as a multiply-add of +0 (a zero product may lose its sign, no value
+// changes): ptxas fuses a packed product into a packed sum that follows, with
+// their roundings written out and contraction off, but not a multiply-add.
+__device__ __forceinline__ float2 mul_(float2 a, float2 b) { return __ffma2_rn(a, b, make_float2(0.0f, 0.0f)); }
 __device__ __forceinline__ float2 fma_(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
 __device__ __forceinline__ float2 sub_(float2 a, float2 b) {
     float2 r;
@@ -171,6 +174,146 @@ __device__ __forceinline__ void collide_pair_each(float2 (&d)[9], float2 (&g)[10
     for (int i = 0; i < 9; ++i) d[i].y = a[i];
 #pragma unroll
     for (int q = 0; q < 10; ++q) g[q].y = b[q];
+}
+
+// ---- the kinetic closures --------------------------------------------------
+// collide_xf, filtered_shift, carati_taus and the moment sums of
+// lbmhd_kinetic.cu (a file compiled without contraction) with every rounding
+// written out: the same operations in the same order, so the same bits.
+__device__ __forceinline__ float recip_(float v) { return __frcp_rn(v); }
+__device__ __forceinline__ float2 recip_(float2 v) { return make_float2(__frcp_rn(v.x), __frcp_rn(v.y)); }
+__device__ __forceinline__ float root_(float v) { return __fsqrt_rn(v); }
+__device__ __forceinline__ float2 root_(float2 v) { return make_float2(__fsqrt_rn(v.x), __fsqrt_rn(v.y)); }
+__device__ __forceinline__ float sign_(float v) { return v > 0.0f ? 1.0f : (v < 0.0f ? -1.0f : 0.0f); }
+__device__ __forceinline__ float2 sign_(float2 v) { return make_float2(sign_(v.x), sign_(v.y)); }
+__device__ __forceinline__ float least_half_(float v) { return v < 0.5f ? 0.5f : v; }
+__device__ __forceinline__ float2 least_half_(float2 v) { return make_float2(least_half_(v.x), least_half_(v.y)); }
+
+// rho, jx, jy, Bx, By of decoded streamed populations.
+template <class T, bool SCALED>
+__device__ __forceinline__ void moments_r(const T (&d)[9], const T (&g)[10], float inv_s, T (&m)[5]) {
+    T drho = add_(add_(add_(add_(d[0], d[1]), add_(d[2], d[3])),
+                       add_(add_(d[4], d[5]), add_(d[6], d[7]))), d[8]);
+    m[1] = add_(add_(sub_(d[1], d[3]), sub_(d[5], d[6])), sub_(d[8], d[7]));
+    m[2] = sub_(add_(sub_(d[2], d[4]), add_(d[5], d[6])), add_(d[7], d[8]));
+    m[3] = add_(add_(add_(g[0], g[2]), add_(g[4], g[6])), g[8]);
+    m[4] = add_(add_(add_(g[1], g[3]), add_(g[5], g[7])), g[9]);
+    if (SCALED) {
+        drho = mul_(inv_s, drho);
+#pragma unroll
+        for (int q = 1; q < 5; ++q) m[q] = mul_(inv_s, m[q]);
+    }
+    m[0] = add_(dup<T>(1.0f), drho);
+}
+
+template <class T>
+__device__ __forceinline__ void filtered_shift_r(const T (&f)[5], const T (&gx)[5], const T (&gy)[5],
+                                                 float d2, T (&sh)[4]) {
+    const T ir = recip_(f[0]);
+    constexpr float twelfth = 1.0f / 12.0f;
+    const T scale = mul_(ir, dup<T>(twelfth));
+    auto dot = [&](int a, int b) { return add_(mul_(gx[a], gx[b]), mul_(gy[a], gy[b])); };
+    T d0[5];
+#pragma unroll
+    for (int a = 0; a < 5; ++a) d0[a] = dot(0, a);
+    auto ratio = [&](int a, int b) {
+        const T in = sub_(add_(mul_(f[a], d0[b]), mul_(f[b], d0[a])), mul_(mul_(mul_(f[a], f[b]), d0[0]), ir));
+        return mul_(sub_(dot(a, b), mul_(in, ir)), scale);
+    };
+    const T rxx = ratio(1, 1), ryy = ratio(2, 2), rxy = ratio(1, 2);
+    sh[0] = mul_(d2, sub_(rxy, mul_(twelfth, dot(3, 4))));
+    sh[1] = mul_(d2, sub_(sub_(rxx, ryy), mul_(twelfth, sub_(dot(3, 3), dot(4, 4)))));
+    sh[2] = mul_(d2, mul_(-3.0f, add_(rxx, ryy)));
+    sh[3] = mul_(d2, sub_(ratio(1, 4), ratio(2, 3)));
+}
+
+// gu, gb: d/dx, d/dy of (u_x, u_y) and (B_x, B_y).
+template <class T>
+__device__ __forceinline__ void carati_taus_r(const T (&gu)[2][2], const T (&gb)[2][2],
+                                              const Coll<float>& c, T (&taus)[2]) {
+    const T svxy = mul_(0.5f, add_(gu[0][1], gu[1][0])), sbxy = mul_(0.5f, add_(gb[0][1], gb[1][0]));
+    const T ss = add_(add_(mul_(gu[0][0], gb[0][0]), mul_(gu[1][1], gb[1][1])), mul_(mul_(2.0f, svxy), sbxy));
+    const T nu_t = mul_(c.cd2, root_(abs_(ss)));
+    const T jw = mul_(sub_(gb[1][0], gb[0][1]), sub_(gu[1][0], gu[0][1]));
+    const T eta_t = mul_(mul_(c.cd2, sign_(jw)), root_(abs_(jw)));
+    taus[0] = add_(dup<T>(c.tn), mul_(3.0f, nu_t));
+    taus[1] = least_half_(add_(dup<T>(c.te), mul_(3.0f, eta_t)));
+}
+
+// KIN: sh = corrections of M_3, M_4, M_7 = M_8, N_y1 (les 2); else sh[0], sh[1]
+// are the relaxation times (les 3).
+template <class T, bool SCALED, bool KIN>
+__device__ __forceinline__ void collide_kin_r(T (&d)[9], T (&g)[10], const Coll<float>& c, const T* sh) {
+    constexpr float k1_3 = 1.0f / 3.0f, k1_6 = 1.0f / 6.0f, k5_3 = 5.0f / 3.0f;
+    constexpr float k1_12 = 1.0f / 12.0f, k1_20 = 1.0f / 20.0f, k1_180 = 1.0f / 180.0f;
+    const T s56 = add_(d[5], d[6]), s78 = add_(d[7], d[8]);
+    const T e56 = sub_(d[5], d[6]), e87 = sub_(d[8], d[7]), e13 = sub_(d[1], d[3]), e24 = sub_(d[2], d[4]);
+    const T dsum9 = add_(add_(add_(add_(d[0], d[1]), add_(d[2], d[3])),
+                              add_(add_(d[4], d[5]), add_(d[6], d[7]))), d[8]);
+    const T jx = add_(add_(e13, e56), e87), jy = sub_(add_(e24, s56), s78);
+    const T rho = SCALED ? fma_(c.inv_s, dsum9, dup<T>(1.0f)) : add_(dup<T>(1.0f), dsum9);
+    const T irho = rcp(rho);
+    const T ux = mul_(jx, irho), uy = mul_(jy, irho);
+    const T bx = add_(add_(add_(g[0], g[2]), add_(g[4], g[6])), g[8]);
+    const T by = add_(add_(add_(g[1], g[3]), add_(g[5], g[7])), g[9]);
+    const T dsum = add_(s56, s78);
+    const T m3 = sub_(e56, e87), m4 = sub_(add_(d[1], d[3]), add_(d[2], d[4]));
+    const T m5 = fma_(-2.0f, e13, add_(e56, e87)), m6 = fma_(-2.0f, e24, sub_(s56, s78));
+    const T m7 = fma_(-5.0f, add_(add_(d[1], d[2]), add_(d[3], d[4])), mul_(4.0f, add_(d[0], dsum)));
+    const T m8 = sub_(mul_(4.0f, d[0]), dsum);
+    const T nbx = neg_(bx), njy = neg_(jy);
+    T j2i = mul_(fma_(jx, jx, mul_(jy, jy)), irho);
+    T q3 = fma_(mul_(jx, jy), irho, mul_(nbx, by));
+    T q4 = fma_(fma_(jx, jx, mul_(njy, jy)), irho, fma_(by, by, mul_(nbx, bx)));
+    T E = fma_(ux, by, mul_(uy, nbx));
+    if (SCALED) {
+        j2i = mul_(c.inv_s, j2i);
+        q3 = mul_(c.inv_s, q3);
+        q4 = mul_(c.inv_s, q4);
+        E = mul_(c.inv_s, E);
+    }
+    if (KIN) {
+        q3 = add_(q3, sh[0]);
+        q4 = add_(q4, sh[1]);
+        E = add_(E, sh[3]);
+    }
+    const T n3 = sub_(m3, q3), n4 = sub_(m4, q4), n5 = add_(m5, jx), n6 = add_(m6, jy);
+    T n7 = fma_(3.0f, j2i, m7), x8 = fma_(k5_3, dsum9, mul_(-3.0f, j2i));
+    if (KIN) {
+        n7 = sub_(n7, sh[2]);
+        x8 = add_(x8, sh[2]);
+    }
+    const T n8 = sub_(m8, x8);
+    const T snu = KIN ? dup<T>(rcp(c.tn)) : rcp(sh[0]);
+    const T nsm = KIN ? dup<T>(-rcp(c.te)) : neg_(rcp(sh[1]));
+    const T s7 = c.s7 > 0.0f ? dup<T>(c.s7) : snu, s8 = c.s8 > 0.0f ? dup<T>(c.s8) : snu;
+    const T a3 = mul_(0.25f, mul_(snu, n3));
+    const T p4 = mul_(snu, n4), a4 = mul_(0.25f, p4), na4 = mul_(-0.25f, p4);
+    const T a5 = mul_(k1_12, mul_(c.s5, n5)), a6 = mul_(k1_12, mul_(c.s6, n6));
+    const T a7 = mul_(k1_180, mul_(s7, n7)), a8 = mul_(k1_20, mul_(s8, n8));
+    const T q78 = sub_(mul_(4.0f, a7), a8);
+    d[0] = fma_(-4.0f, add_(a7, a8), d[0]);
+    d[1] = add_(d[1], fma_(5.0f, a7, fma_(2.0f, a5, na4)));
+    d[2] = add_(d[2], fma_(5.0f, a7, fma_(2.0f, a6, a4)));
+    d[3] = add_(d[3], fma_(5.0f, a7, fma_(-2.0f, a5, na4)));
+    d[4] = add_(d[4], fma_(5.0f, a7, fma_(-2.0f, a6, a4)));
+    const T D = sub_(a3, a5), H = sub_(a6, q78);
+    d[5] = sub_(d[5], add_(add_(a3, a5), add_(a6, q78)));
+    d[6] = sub_(d[6], sub_(sub_(a6, a3), sub_(a5, q78)));
+    d[7] = sub_(d[7], sub_(D, H));
+    d[8] = add_(d[8], add_(D, H));
+    const T e3 = mul_(3.0f, E), bx6 = mul_(k1_6, bx), by6 = mul_(k1_6, by);
+    auto relax = [&](int q, T eq) { g[q] = fma_(nsm, sub_(g[q], eq), g[q]); };
+    relax(0, mul_(k1_3, bx));
+    relax(1, mul_(k1_3, by));
+    relax(2, bx6);
+    relax(3, mul_(k1_6, add_(by, e3)));
+    relax(4, mul_(k1_6, sub_(bx, e3)));
+    relax(5, by6);
+    relax(6, bx6);
+    relax(7, mul_(k1_6, sub_(by, e3)));
+    relax(8, mul_(k1_6, add_(bx, e3)));
+    relax(9, by6);
 }
 
 }  // namespace lbmhd

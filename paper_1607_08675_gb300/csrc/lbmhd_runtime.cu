@@ -158,16 +158,18 @@ cudaError_t launch_one(lbmhd_t* h, const void* src, void* dst) {
 }
 
 // Steps of the next launch when `left` steps follow each other: the passes
-// of at most kPipeSteps steps are kept even (5 = 3 + 2, 6 = 3 + 3), so that
+// of at most h->pipe steps are kept even (5 = 3 + 2, 6 = 3 + 3), so that
 // only a single step on its own takes the one-step kernel.
 int next_steps(const lbmhd_t* h, int left) {
     if (!h->pipe || left < 2) return 1;
-    const int passes = (left + kPipeSteps - 1) / kPipeSteps;
+    const int passes = (left + h->pipe - 1) / h->pipe;
     return (left + passes - 1) / passes;
 }
 
 // One launch of k steps from src to dst.
 cudaError_t launch_steps(lbmhd_t* h, int k, const void* src, void* dst) {
+    if (k > 1 && h->coll.kin)
+        return launch_kin_pipe(h->p.precision, src, dst, h->geom, h->coll, h->sm_count, h->stream);
     if (k > 1)
         return launch_pipe(h->p.precision, k, src, dst, h->geom, h->coll, h->sm_count, h->stream);
     return launch_one(h, src, dst);
@@ -287,7 +289,7 @@ int lbmhd_create(int nx, int ny, const lbmhd_params* p, lbmhd_t** out) {
                : h->vec == 4 || p->precision == LBMHD_FP64 ? 64
                : p->precision == LBMHD_FF && !ff_small ? 256 : 128;
     h->tma_w = 0;
-    h->pipe = h->coll.kin == 0 && pipe_ok(p->precision, (long long)nx * ny);
+    h->pipe = pipe_steps(p->precision, (long long)nx * ny, h->coll.kin != 0);
     // Kinetic steps: the fused kernel where it is faster (measured at 8192^2
     // / 4096^2, MLUPS fused vs two-pass: FP32 les 2 33.5K vs 23.7K, les 3
     // 37.1K vs 22.3K; FP16 38.9K vs 26.6K; FF les 3 8.2K vs 7.2K), the

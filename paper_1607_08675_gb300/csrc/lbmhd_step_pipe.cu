@@ -58,7 +58,9 @@ namespace {
 // where a launch is mostly latency and one for four steps takes less than
 // four (FP32 64^2 2.23 / 1.77, 128^2 2.57 / 1.90, 256^2 3.16 / 3.19).
 // Between them the rows that segments share cost as much as the passes save
-// (FP32 512^2 5.8 / 6.3).
+// (FP32 512^2 5.8 / 6.3).  The kinetic closures, two steps per pass: only the
+// large ones (les 2 FP32, us per step, one-step / this: 128^2 2.9 / 3.6, 512^2
+// 11.4 / 12.2, 1024^2 39.4 / 28.3).
 constexpr long long kPipeBytes = 80LL << 20;
 constexpr long long kPipeSmall = 32768;
 
@@ -88,11 +90,9 @@ __device__ __forceinline__ unsigned stream1(unsigned v) {
     return __byte_perm(v, __shfl_down_sync(0xffffffffu, v, 1), 0x5432);
 }
 
-// Both columns of a pair through the collision, stored form to stored form.
+// A row's pairs from their stored form, and back.
 template <int P>
-__device__ __forceinline__ void collide_pair(typename PairOf<P>::T (&z)[kPlanes], const Coll<float>& c) {
-    constexpr bool SC = Fmt<P>::kScaled, ABS = P == P_FP32;
-    float2 d[9], g[10];
+__device__ __forceinline__ void unpack(const typename PairOf<P>::T (&z)[kPlanes], float2 (&d)[9], float2 (&g)[10]) {
 #pragma unroll
     for (int p = 0; p < kPlanes; ++p) {
         float2 v;
@@ -102,7 +102,9 @@ __device__ __forceinline__ void collide_pair(typename PairOf<P>::T (&z)[kPlanes]
         if (p < 9) d[p] = v;
         else g[p - 9] = v;
     }
-    collide_r<float2, SC, ABS>(d, g, c);
+}
+template <int P>
+__device__ __forceinline__ void pack(const float2 (&d)[9], const float2 (&g)[10], typename PairOf<P>::T (&z)[kPlanes]) {
 #pragma unroll
     for (int p = 0; p < kPlanes; ++p) {
         float2 v = p < 9 ? d[p] : g[p - 9];
@@ -114,6 +116,15 @@ __device__ __forceinline__ void collide_pair(typename PairOf<P>::T (&z)[kPlanes]
             z[p] = v;
         }
     }
+}
+
+// Both columns of a pair through the collision, stored form to stored form.
+template <int P>
+__device__ __forceinline__ void collide_pair(typename PairOf<P>::T (&z)[kPlanes], const Coll<float>& c) {
+    float2 d[9], g[10];
+    unpack<P>(z, d, g);
+    collide_r<float2, Fmt<P>::kScaled, P == P_FP32>(d, g, c);
+    pack<P>(d, g, z);
 }
 
 // Place of plane p among the planes that do not move along y.
@@ -134,6 +145,62 @@ struct PipeShape {
 // there: 72 G); FP16, whose history is packed, 128 at every S.
 __host__ __device__ constexpr int pipe_warps(int prec, int steps) {
     return prec == P_FP16_DEV || steps == 2 ? 4 : (steps == 3 ? 3 : 2);
+}
+
+// The populations that stream along y into row r0 of the lane's columns xa, xb
+// (fetched ahead into pre by cp.async, or into z), and on to the next row.
+template <int P, bool AL, int N>
+__device__ __forceinline__ void fetch_row(const typename Fmt<P>::S* __restrict__ src, int nx, long long ps,
+                                          int xa, int xb, int& rm, int& r0, int& rp, int ny,
+                                          typename PairOf<P>::T (&pre)[N][32],
+                                          typename PairOf<P>::T (&z)[kPlanes]) {
+    using T = typename Fmt<P>::S;
+    const int lane = threadIdx.x;
+    const unsigned om = (unsigned)rm * (unsigned)nx, o0 = (unsigned)r0 * (unsigned)nx,
+                   op = (unsigned)rp * (unsigned)nx;
+#pragma unroll
+    for (int p = 0; p < kPlanes; ++p) {
+        const unsigned row = plane_cy(p) == 0 ? o0 : (plane_cy(p) > 0 ? om : op);
+        const T* base = src + p * ps;
+        if constexpr (AL) cp_async_small<2 * sizeof(T)>(&pre[p][lane], base + (row + xa));
+        else if constexpr (P != P_FP16_DEV) {
+            cp_async_small<4>(&pre[p][lane].x, base + (row + xa));
+            cp_async_small<4>(&pre[p][lane].y, base + (row + xb));
+        } else {
+            z[p] = (unsigned)base[row + xa] | (unsigned)base[row + xb] << 16;
+        }
+    }
+    if (AL || P != P_FP16_DEV) cp_async_commit();
+    rm = r0;
+    r0 = rp;
+    rp = rp + 1 == ny ? 0 : rp + 1;
+}
+
+// A row streamed along x.
+template <int P>
+__device__ __forceinline__ void stream_row(typename PairOf<P>::T (&v)[kPlanes]) {
+#pragma unroll
+    for (int p = 0; p < kPlanes; ++p)
+        v[p] = plane_cx(p) == 0 ? v[p] : (plane_cx(p) > 0 ? stream1<1>(v[p]) : stream1<-1>(v[p]));
+}
+
+template <int P, bool AL>
+__device__ __forceinline__ void store_row(typename Fmt<P>::S* __restrict__ dst, long long ps, unsigned orow,
+                                          bool outb, const typename PairOf<P>::T (&z)[kPlanes]) {
+    using T = typename Fmt<P>::S;
+#pragma unroll
+    for (int p = 0; p < kPlanes; ++p) {
+        T* o = dst + p * ps + orow;
+        if constexpr (AL) {
+            *reinterpret_cast<typename PairOf<P>::T*>(o) = z[p];
+        } else if constexpr (P == P_FP16_DEV) {
+            o[0] = (T)z[p];
+            if (outb) o[1] = (T)(z[p] >> 16);
+        } else {
+            o[0] = z[p].x;
+            if (outb) o[1] = z[p].y;
+        }
+    }
 }
 
 // The shared memory of one warp.
@@ -172,38 +239,8 @@ __device__ __forceinline__ void pipe_body(const typename Fmt<P>::S* __restrict__
     r0 = rm + 1 == ny ? 0 : rm + 1;
     rp = r0 + 1 == ny ? 0 : r0 + 1;
 
-    // the populations that stream along y into row r0 of the lane's columns
-    auto fetch = [&](Q(&z)[kPlanes]) {
-        const unsigned om = (unsigned)rm * (unsigned)nx, o0 = (unsigned)r0 * (unsigned)nx,
-                       op = (unsigned)rp * (unsigned)nx;
-#pragma unroll
-        for (int p = 0; p < kPlanes; ++p) {
-            const unsigned row = plane_cy(p) == 0 ? o0 : (plane_cy(p) > 0 ? om : op);
-            const T* base = src + p * ps;
-            if constexpr (PF) {
-                if (AL) cp_async_small<2 * sizeof(T)>(&pre[p][lane], base + (row + xa));
-                else if constexpr (P != P_FP16_DEV) {
-                    cp_async_small<4>(&pre[p][lane].x, base + (row + xa));
-                    cp_async_small<4>(&pre[p][lane].y, base + (row + xb));
-                }
-            } else if constexpr (P == P_FP16_DEV) {
-                if (AL) z[p] = *reinterpret_cast<const unsigned*>(base + (row + xa));
-                else z[p] = (unsigned)base[row + xa] | (unsigned)base[row + xb] << 16;
-            } else {
-                if (AL) z[p] = *reinterpret_cast<const float2*>(base + (row + xa));
-                else z[p] = make_float2(base[row + xa], base[row + xb]);
-            }
-        }
-        if (PF) cp_async_commit();
-        rm = r0;
-        r0 = rp;
-        rp = rp + 1 == ny ? 0 : rp + 1;
-    };
-    auto stream = [&](Q(&v)[kPlanes]) {
-#pragma unroll
-        for (int p = 0; p < kPlanes; ++p)
-            v[p] = plane_cx(p) == 0 ? v[p] : (plane_cx(p) > 0 ? stream1<1>(v[p]) : stream1<-1>(v[p]));
-    };
+    auto fetch = [&](Q(&z)[kPlanes]) { fetch_row<P, AL>(src, nx, ps, xa, xb, rm, r0, rp, ny, pre, z); };
+    auto stream = [&](Q(&v)[kPlanes]) { stream_row<P>(v); };
 
     Q h1[S - 1][kPlanes], h2[S - 1][kPlanes];  // c_y > 0: the last row and the one before
     const int n = y1 - y0 + 2 * (S - 1);
@@ -250,25 +287,177 @@ __device__ __forceinline__ void pipe_body(const typename Fmt<P>::S* __restrict__
             for (int p = 0; p < kPlanes; ++p) z[p] = w[p];
         }
         if (done) continue;
-        if (outa) {
+        if (outa) store_row<P, AL>(dst, ps, orow, outb, z);
+        orow += (unsigned)nx;
+    }
+}
+
+// ---- two steps of a kinetic closure (les 2, 3) per pass ---------------------
+// A step of these closures needs the conserved moments of the streamed
+// populations at the four neighbours, so each of the two steps keeps its
+// last streamed row (in shared memory) and the moments of its last two rows
+// (in registers), and collides a row when the next one has been streamed:
+// one more row of lag and one more halo column on each side per step than
+// above.  Measured on GB300 (us per step, the one-step fused kernel / this):
+// 8192^2 FP32 les 2 1735 / 1116, les 3 1737 / 1098; FP16 les 2 1521 / 1081, les 3
+// 1517 / 955; 4096^2 FP32 les 2 448 / 293.  The one-step kernel ran at 0.87 of
+// the copy bandwidth at 152 B per node; this one is bound by issue and
+// latency at two warps per scheduler.
+template <int P, bool AL>
+struct KinShared {
+    using Q = typename PairOf<P>::T;
+    static constexpr bool PF = AL || P != P_FP16_DEV;
+    Q pre[PF ? kPlanes : 1][32];
+    Q row[2][kPlanes][32];  // each step's last streamed row
+    Q keep[9][32];          // the first step's last result, c_y = 0
+};
+constexpr int kKinHalo = 4, kKinUseful = 64 - 2 * kKinHalo;
+
+__device__ __forceinline__ float2 west(float2 v) { return stream1<1>(v); }   // values at x - 1
+__device__ __forceinline__ float2 east(float2 v) { return stream1<-1>(v); }  // at x + 1
+
+// The closure's fields of a streamed row: rho, j, B (les 2) or u, B (les 3).
+template <int P, int MODE>
+__device__ __forceinline__ void kin_fields(const typename PairOf<P>::T (&z)[kPlanes], const Coll<float>& c,
+                                           float2 (&m)[MODE == 2 ? 5 : 4]) {
+    float2 d[9], g[10], a[5];
+    unpack<P>(z, d, g);
+    moments_r<float2, Fmt<P>::kScaled>(d, g, c.inv_s, a);
+    if constexpr (MODE == 2) {
 #pragma unroll
-            for (int p = 0; p < kPlanes; ++p) {
-                T* o = dst + p * ps + orow;
-                if constexpr (P == P_FP16_DEV) {
-                    if (AL) *reinterpret_cast<unsigned*>(o) = z[p];
-                    else {
-                        o[0] = (T)z[p];
-                        if (outb) o[1] = (T)(z[p] >> 16);
-                    }
-                } else {
-                    if (AL) *reinterpret_cast<float2*>(o) = z[p];
-                    else {
-                        o[0] = z[p].x;
-                        if (outb) o[1] = z[p].y;
+        for (int q = 0; q < 5; ++q) m[q] = a[q];
+    } else {
+        const float2 ir = recip_(a[0]);
+        m[0] = mul_(a[1], ir);
+        m[1] = mul_(a[2], ir);
+        m[2] = a[3];
+        m[3] = a[4];
+    }
+}
+
+// A streamed row collided with the fields of the row below (lo), its own (at)
+// and the row above (hi).
+template <int P, int MODE>
+__device__ __forceinline__ void kin_collide(typename PairOf<P>::T (&z)[kPlanes],
+                                            const float2 (&lo)[MODE == 2 ? 5 : 4],
+                                            const float2 (&at)[MODE == 2 ? 5 : 4],
+                                            const float2 (&hi)[MODE == 2 ? 5 : 4], const Coll<float>& c) {
+    constexpr int NF = MODE == 2 ? 5 : 4;
+    constexpr bool SC = Fmt<P>::kScaled;
+    float2 gx[NF], gy[NF];
+#pragma unroll
+    for (int q = 0; q < NF; ++q) {
+        gx[q] = mul_(0.5f, sub_(east(at[q]), west(at[q])));
+        gy[q] = mul_(0.5f, sub_(hi[q], lo[q]));
+    }
+    float2 d[9], g[10];
+    if constexpr (MODE == 2) {
+        float2 sh[4];
+        filtered_shift_r<float2>(at, gx, gy, c.d2, sh);
+        if (SC)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) sh[q] = mul_(c.scl, sh[q]);
+        unpack<P>(z, d, g);
+        collide_kin_r<float2, SC, true>(d, g, c, sh);
+    } else {
+        const float2 gu[2][2] = {{gx[0], gy[0]}, {gx[1], gy[1]}}, gb[2][2] = {{gx[2], gy[2]}, {gx[3], gy[3]}};
+        float2 taus[2];
+        carati_taus_r<float2>(gu, gb, c, taus);
+        unpack<P>(z, d, g);
+        collide_kin_r<float2, SC, false>(d, g, c, taus);
+    }
+    pack<P>(d, g, z);
+}
+
+// Warps per scheduler: two for FP32 (222 registers; at 168 it spills, 1753 us
+// per step), three for FP16.
+constexpr int kin_pipe_warps(int prec) { return prec == P_FP16_DEV ? 3 : 2; }
+template <int P, int MODE, bool AL>
+__global__ void __launch_bounds__(32, 4 * kin_pipe_warps(P))
+    kin_pipe_kernel(const typename Fmt<P>::S* __restrict__ src, typename Fmt<P>::S* __restrict__ dst,
+                    int nx, int ny, long long ps, int strips, int seglen, Coll<float> c) {
+    using T = typename Fmt<P>::S;
+    using Q = typename PairOf<P>::T;
+    constexpr int NF = MODE == 2 ? 5 : 4;
+    constexpr bool PF = KinShared<P, AL>::PF;
+    __shared__ KinShared<P, AL> sh;
+    const int strip = (int)(blockIdx.x % (unsigned)strips), seg = (int)(blockIdx.x / (unsigned)strips);
+    const int y0 = seg * seglen, y1 = min(y0 + seglen, ny);
+    const int lane = threadIdx.x;
+    const int x = strip * kKinUseful - kKinHalo + 2 * lane;
+    int xa = x % nx;
+    if (xa < 0) xa += nx;
+    const int xb = xa + 1 == nx ? 0 : xa + 1;
+    const bool outa = x >= strip * kKinUseful && x < strip * kKinUseful + kKinUseful && x < nx;
+    const bool outb = outa && x + 1 < nx;
+    int rm = (y0 - 4) % ny, r0, rp;  // the first streamed row is y0 - 3
+    if (rm < 0) rm += ny;
+    r0 = rm + 1 == ny ? 0 : rm + 1;
+    rp = r0 + 1 == ny ? 0 : r0 + 1;
+    auto fetch = [&](Q(&z)[kPlanes]) { fetch_row<P, AL>(src, nx, ps, xa, xb, rm, r0, rp, ny, sh.pre, z); };
+
+    Q h1[kPlanes], h2[kPlanes];           // the first step's results, c_y > 0
+    float2 ma[2][NF], mb[2][NF], mc[NF];  // fields of each step's last two rows, and the new one
+#pragma unroll
+    for (int k = 0; k < 2; ++k)
+#pragma unroll
+        for (int q = 0; q < NF; ++q) ma[k][q] = mb[k][q] = make_float2(1.0f, 1.0f);
+    const int n = y1 - y0 + 6;
+    unsigned orow = (unsigned)y0 * (unsigned)nx + (unsigned)x;
+    Q z[kPlanes];
+    if (PF) fetch(z);
+#pragma unroll 1
+    for (int it = 0; it < n; ++it) {
+        if (PF) {
+            cp_async_wait<0>();
+#pragma unroll
+            for (int p = 0; p < kPlanes; ++p) z[p] = sh.pre[p][lane];
+            stream_row<P>(z);
+            if (it + 1 < n) fetch(z);
+        } else {
+            fetch(z);
+            stream_row<P>(z);
+        }
+        bool done = false;
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            if (done) continue;
+            if (k == 1) {  // the second step's streamed row from the first one's results
+                stream_row<P>(z);
+#pragma unroll
+                for (int p = 0; p < kPlanes; ++p) {
+                    const Q v = z[p];
+                    if (plane_cy(p) == 0) {
+                        z[p] = sh.keep[keep_slot(p)][lane];
+                        sh.keep[keep_slot(p)][lane] = v;
+                    } else if (plane_cy(p) > 0) {
+                        z[p] = h2[p];
+                        h2[p] = h1[p];
+                        h1[p] = v;
                     }
                 }
+                if (it < 4) {
+                    done = true;
+                    continue;
+                }
+            }
+            kin_fields<P, MODE>(z, c, mc);
+#pragma unroll
+            for (int p = 0; p < kPlanes; ++p) {  // the row before this one comes out
+                const Q v = z[p];
+                z[p] = sh.row[k][p][lane];
+                sh.row[k][p][lane] = v;
+            }
+            if (it >= 4 * k + 2) kin_collide<P, MODE>(z, ma[k], mb[k], mc, c);
+            else done = true;
+#pragma unroll
+            for (int q = 0; q < NF; ++q) {
+                ma[k][q] = mb[k][q];
+                mb[k][q] = mc[q];
             }
         }
+        if (done) continue;
+        if (outa) store_row<P, AL>(dst, ps, orow, outb, z);
         orow += (unsigned)nx;
     }
 }
@@ -357,11 +546,39 @@ cudaError_t launch_pipe_p(int steps, const void* src, void* dst, const Geom& g, 
     return cudaErrorInvalidValue;
 }
 
+template <int P>
+cudaError_t launch_kin_pipe_p(const void* src, void* dst, const Geom& g, const HostColl& hc, int sm_count,
+                              cudaStream_t st) {
+    using T = typename Fmt<P>::S;
+    const int strips = (g.nx + kKinUseful - 1) / kKinUseful;
+    const int seglen = best_seglen(4, kin_pipe_warps(P), g.ny, sm_count, [&](int len) {
+        return (long long)strips * ((g.ny + len - 1) / len);
+    });
+    const bool al = g.nx % 2 == 0;
+    auto k = hc.kin == 3 ? (al ? kin_pipe_kernel<P, 3, true> : kin_pipe_kernel<P, 3, false>)
+                         : (al ? kin_pipe_kernel<P, 2, true> : kin_pipe_kernel<P, 2, false>);
+    k<<<(unsigned)strips * (unsigned)((g.ny + seglen - 1) / seglen), 32, 0, st>>>(
+        (const T*)src, (T*)dst, g.nx, g.ny, g.ps, strips, seglen, coll_for_prec<float>(hc, P));
+    return cudaGetLastError();
+}
+
 }  // namespace
 
-bool pipe_ok(int prec, long long nodes) {
-    if (prec != P_FP32 && prec != P_FP32_DEV && prec != P_FP16_DEV) return false;
-    return nodes <= kPipeSmall || 2 * kPlanes * (long long)storage_bytes(prec) * nodes >= kPipeBytes;
+cudaError_t launch_kin_pipe(int prec, const void* src, void* dst, const Geom& g, const HostColl& c,
+                            int sm_count, cudaStream_t st) {
+    switch (prec) {
+        case P_FP32: return launch_kin_pipe_p<P_FP32>(src, dst, g, c, sm_count, st);
+        case P_FP32_DEV: return launch_kin_pipe_p<P_FP32_DEV>(src, dst, g, c, sm_count, st);
+        case P_FP16_DEV: return launch_kin_pipe_p<P_FP16_DEV>(src, dst, g, c, sm_count, st);
+    }
+    return cudaErrorInvalidValue;
+}
+
+int pipe_steps(int prec, long long nodes, bool kin) {
+    if (prec != P_FP32 && prec != P_FP32_DEV && prec != P_FP16_DEV) return 0;
+    const bool large = 2 * kPlanes * (long long)storage_bytes(prec) * nodes >= kPipeBytes;
+    if (kin) return large ? kKinPipeSteps : 0;
+    return large || nodes <= kPipeSmall ? kPipeSteps : 0;
 }
 
 int batch_pipe_plan(int prec, int nruns, const int* nx, const int* ny, int sm_count, int* strips) {

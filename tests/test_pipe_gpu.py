@@ -60,6 +60,24 @@ def test_several_steps_per_launch_equal_single_steps(L, prec, shape):
             assert launches == 8
 
 
+# about 1.2 M nodes, where the kinetic closures take two steps per pass: one and
+# two nodes wide or high, and around the 56 columns that a strip stores
+THIN = [(1, 1200000), (1200000, 1), (2, 600000), (400001, 3), (55, 21819), (57, 21053), (113, 10620)]
+
+
+@pytest.mark.parametrize("prec", ["fp32", "fp32_dev", "fp16_dev"])
+@pytest.mark.parametrize("shape", THIN)
+def test_two_steps_of_a_kinetic_closure_equal_single_steps(L, prec, shape):
+    """les 2 and 3, two steps per launch, against the one-step fused kernel
+    (vec 1) bit for bit."""
+    fields = inputs.orszag_tang(*shape, seed=3, amp=1e-3)
+    for les in (2, 3):
+        got, launches = raw(L, shape, fields, prec, les, (2, 3), False)
+        ref, one = raw(L, shape, fields, prec, les, (2, 3), True)
+        assert np.array_equal(got, ref), (shape, les)
+        assert one == 5 and launches == 3
+
+
 def test_several_steps_per_launch_with_tied_rates_and_graph_replay(L):
     """Rates s_7, s_8 tied to the local s_nu and a run long enough for graph
     replay, in calls that leave the buffers in either parity."""
