@@ -35,6 +35,7 @@
 
 #include "lbmhd_internal.h"
 #include "lbmhd_narrow.cuh"
+#include "lbmhd_pdl.cuh"
 #include "lbmhd_step_body.cuh"
 
 namespace lbmhd {
@@ -260,6 +261,7 @@ __global__ void __launch_bounds__(kAdjBlock) adj_step_kernel(
     typename Fmt<P>::R* __restrict__ lout, int nx, int ny, long long ps,
     Coll<typename Fmt<P>::R> c, float inv_scale, double* __restrict__ partials) {
     using R = typename Fmt<P>::R;
+    after_previous();
     const long long n = (long long)nx * ny;
     // per-thread sensitivity sums: FP64 for FP64 storage; double-word for
     // the FP32 forms, which keeps FP64 instructions out of the node loop
@@ -479,12 +481,9 @@ cudaError_t run_adj_step(const lbmhd_t* h, const void* x, const void* lin, void*
     using R = typename Fmt<P>::R;
     const long long n = (long long)h->geom.nx * h->geom.ny;
     const unsigned grid = adj_grid(n);
-    adj_step_kernel<P><<<grid, kAdjBlock, 0, h->stream>>>(
-        (const S*)x, (const R*)lin, (R*)lout, h->geom.nx, h->geom.ny, h->geom.ps,
-        coll_t<R>(h->coll), h->coll.inv_scale, partials);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    return cudaGetLastError();
+    return launch_after(adj_step_kernel<P>, grid, kAdjBlock, h->stream, (const S*)x, (const R*)lin,
+                        (R*)lout, h->geom.nx, h->geom.ny, h->geom.ps, coll_t<R>(h->coll),
+                        h->coll.inv_scale, partials);
 }
 
 template <int P>

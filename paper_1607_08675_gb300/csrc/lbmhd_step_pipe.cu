@@ -45,6 +45,7 @@
 #include "lbmhd_cp_async.cuh"
 #include "lbmhd_internal.h"
 #include "lbmhd_pair.cuh"
+#include "lbmhd_pdl.cuh"
 #include "lbmhd_step_body.cuh"
 
 namespace lbmhd {
@@ -381,6 +382,7 @@ __global__ void __launch_bounds__(32, 4 * kin_pipe_warps(P))
     constexpr int NF = MODE == 2 ? 5 : 4;
     constexpr bool PF = KinShared<P, AL>::PF;
     __shared__ KinShared<P, AL> sh;
+    after_previous();
     const int strip = (int)(blockIdx.x % (unsigned)strips), seg = (int)(blockIdx.x / (unsigned)strips);
     const int y0 = seg * seglen, y1 = min(y0 + seglen, ny);
     const int lane = threadIdx.x;
@@ -467,6 +469,7 @@ __global__ void __launch_bounds__(32, 4 * pipe_warps(P, S))
     pipe_kernel(const typename Fmt<P>::S* __restrict__ src, typename Fmt<P>::S* __restrict__ dst,
                 int nx, int ny, long long ps, int strips, int seglen, Coll<float> c) {
     __shared__ PipeShared<P, S, AL> sh;
+    after_previous();
     const int strip = (int)(blockIdx.x % (unsigned)strips), seg = (int)(blockIdx.x / (unsigned)strips);
     const int y0 = seg * seglen;
     pipe_body<P, S, AL>(src, dst, nx, ny, ps, strip, y0, min(y0 + seglen, ny), c, sh);
@@ -482,6 +485,7 @@ __global__ void __launch_bounds__(32, 4 * batch_pipe_warps(P))
     batch_pipe_kernel(const RunDev<float>* __restrict__ runs, const int* __restrict__ unit_run,
                       const typename Fmt<P>::S* __restrict__ src, typename Fmt<P>::S* __restrict__ dst) {
     __shared__ PipeShared<P, kPipeSteps, AL> sh;
+    after_previous();
     const RunDev<float>& rd = runs[unit_run[blockIdx.x]];
     const int l = (int)(blockIdx.x - rd.punit0);
     const int strip = l % rd.pstrips, y0 = l / rd.pstrips * rd.pseglen;
@@ -529,9 +533,8 @@ cudaError_t launch_pipe_t(const void* src, void* dst, const Geom& g, const HostC
         return (long long)strips * ((g.ny + len - 1) / len);
     });
     const int nseg = (g.ny + seglen - 1) / seglen;
-    pipe_kernel<P, S, AL><<<(unsigned)strips * (unsigned)nseg, 32, 0, st>>>(
-        (const T*)src, (T*)dst, g.nx, g.ny, g.ps, strips, seglen, coll_for_prec<float>(hc, P));
-    return cudaGetLastError();
+    return launch_after(pipe_kernel<P, S, AL>, (unsigned)strips * (unsigned)nseg, 32, st, (const T*)src,
+                        (T*)dst, g.nx, g.ny, g.ps, strips, seglen, coll_for_prec<float>(hc, P));
 }
 
 template <int P>
@@ -557,9 +560,8 @@ cudaError_t launch_kin_pipe_p(const void* src, void* dst, const Geom& g, const H
     const bool al = g.nx % 2 == 0;
     auto k = hc.kin == 3 ? (al ? kin_pipe_kernel<P, 3, true> : kin_pipe_kernel<P, 3, false>)
                          : (al ? kin_pipe_kernel<P, 2, true> : kin_pipe_kernel<P, 2, false>);
-    k<<<(unsigned)strips * (unsigned)((g.ny + seglen - 1) / seglen), 32, 0, st>>>(
-        (const T*)src, (T*)dst, g.nx, g.ny, g.ps, strips, seglen, coll_for_prec<float>(hc, P));
-    return cudaGetLastError();
+    return launch_after(k, (unsigned)strips * (unsigned)((g.ny + seglen - 1) / seglen), 32, st,
+                        (const T*)src, (T*)dst, g.nx, g.ny, g.ps, strips, seglen, coll_for_prec<float>(hc, P));
 }
 
 }  // namespace
@@ -600,17 +602,15 @@ cudaError_t launch_batch_pipe(int prec, bool even, const void* runs, const int* 
     const RunDev<float>* rd = (const RunDev<float>*)runs;
 #define LBMHD_BP(P)                                                                           \
     case P:                                                                                   \
-        (even ? batch_pipe_kernel<P, true> : batch_pipe_kernel<P, false>)<<<nunits, 32, 0, st>>>( \
-            rd, unit_run, (const Fmt<P>::S*)src, (Fmt<P>::S*)dst);                            \
-        break;
+        return launch_after(even ? batch_pipe_kernel<P, true> : batch_pipe_kernel<P, false>, nunits, \
+                            32, st, rd, unit_run, (const Fmt<P>::S*)src, (Fmt<P>::S*)dst);
     switch (prec) {
         LBMHD_BP(P_FP32)
         LBMHD_BP(P_FP32_DEV)
         LBMHD_BP(P_FP16_DEV)
-        default: return cudaErrorInvalidValue;
     }
 #undef LBMHD_BP
-    return cudaGetLastError();
+    return cudaErrorInvalidValue;
 }
 
 cudaError_t launch_pipe(int prec, int steps, const void* src, void* dst, const Geom& g,
