@@ -5,10 +5,11 @@ the HBM roofline).
 Workload (default): decaying 2D MHD turbulence on an 8192 x 8192 periodic
 lattice (random-phase modes 4 <= |k| <= 8, rms 0.04, C_S = 0.1,
 tau = 0.51), FP32 storage and arithmetic, 500 steps timed after warm-up.
-The state (10 GB per buffer) is far larger than L2, so no flush is needed
-between steps.  The same run also times, on the same lattice, the paper's
-kinetic LES (les = 2; the fused one-launch kernel and the two-pass
-kernels), the FP64, double-word (FF), FP32-deviation and FP16-deviation
+A launch takes up to four steps in one pass over the state; the roofline
+fraction is that of a pass.  The state (5.1 GB per buffer) is far larger
+than L2, so no flush is needed between launches.  The same run also times,
+on the same lattice, the paper's kinetic LES (les = 2; two steps per pass,
+the fused one-step kernel and the two-pass kernels), the FP64, double-word (FF), FP32-deviation and FP16-deviation
 storage forms (fewer steps), an end-to-end pass through the host C ABI
 (host fields in, host moments out), the 256-run ensemble, the adjoint
 (gradients), and the CPU oracle on a bounded sample.
@@ -250,7 +251,7 @@ def kernel_source_hash() -> str:
     import hashlib
 
     h = hashlib.sha256()
-    for f in ("lbmhd_step.cu", "lbmhd_step_body.cuh", "lbmhd_device.cuh"):
+    for f in ("lbmhd_step_pipe.cu", "lbmhd_pair.cuh", "lbmhd_device.cuh"):
         with open(os.path.join(ROOT, "paper_1607_08675_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]
@@ -372,14 +373,14 @@ def run_batched(L, args, stream, rank, hbm, barrier, max_over_ranks):
                "hbm_frac": cells * ksteps * 152 / tk_batch / 1e9 / hbm,
                "kernel": "fused" if kshape[0] == 1 else "two-pass",
                "note": "les=2 ensemble: the fused kernel over every run's strip-segments, one "
-                       "launch per step (152 B/node), vs the runs one by one with the fused "
-                       "single-lattice kernel"}
+                       "launch per step (152 B/node), vs the runs one by one with their own "
+                       "default kernels (two steps per pass for the large ones)"}
     return {"MLUPS": mlups, "sequential_MLUPS": world * cells * steps / t_seq / 1e6,
             "kinetic_les": kinetic,
             "speedup": t_seq / t_batch, "runs": len(runs), "cells": cells, "steps": steps,
             "launch": {"vec": shape[0], "block": shape[1], "steps_per_launch": shape[2]},
             "autotune_trial_MLUPS": tuned, "persistent_launches": int(launches),
-            "hbm_frac": cells * steps * 152 / t_batch / 1e9 / hbm,
+            "hbm_frac_at_one_pass_per_step": cells * steps * 152 / t_batch / 1e9 / hbm,
             "sizes": {str(k): nx.count(k) for k in sorted(set(nx))}}
 
 
@@ -637,7 +638,9 @@ def run_ours(args):
     cells = n * n
     value = job_rate(world, cells, args.steps, dt)
     bpc = L.lbmhd_bytes_per_cell(prec)
-    per_launch_s = (e0.elapsed_time(e1) / 1e3) / args.steps
+    # a launch passes over the state once (bytes_per_cell per node) and advances
+    # it by up to four steps
+    per_launch_s = (e0.elapsed_time(e1) / 1e3) / launches
     achieved = bpc * cells / per_launch_s / 1e9
     L.lbmhd_destroy(h)
     del h
@@ -645,16 +648,19 @@ def run_ours(args):
     # ---- other storage forms on the same lattice ---------------------------
     variants = {}
     if not args.no_variants:
-        # the paper's kinetic LES, FP32: the fused one-launch kernel (default;
-        # algorithmic bytes per node 19 reads + 19 writes, as a plain step) and
-        # the two-pass kernels (19 reads + 5 writes, 19 + 5 reads + 19 writes)
-        # and the cross-helicity closure (les = 3) with the fused kernel
-        for kname, kles, kvec, kbytes in (("fp32_kinetic_les", 2, 1, 152),
+        # the paper's kinetic LES, FP32: the fused one-step kernel (algorithmic
+        # bytes per node 19 reads + 19 writes, as a plain step), the two-pass
+        # kernels (19 reads + 5 writes, 19 + 5 reads + 19 writes)
+        # and the cross-helicity closure (les = 3); kvec None: the default, two
+        # steps per pass (76 B per node and step)
+        for kname, kles, kvec, kbytes in (("fp32_kinetic_les", 2, None, 76),
+                                          ("fp32_kinetic_les_one_step", 2, 1, 152),
                                           ("fp32_kinetic_les_two_pass", 2, 0, 268),
-                                          ("fp32_cross_helicity", 3, 1, 152)):
+                                          ("fp32_cross_helicity", 3, None, 76)):
             hk = L.lbmhd_create(n, n, L.lbmhd_params_default(
                 precision="fp32", **dict(kw, les=kles, delta=2.0)))
-            L.lbmhd_set_launch(hk, kvec, 256)
+            if kvec is not None:
+                L.lbmhd_set_launch(hk, kvec, 256)
             L.lbmhd_init(hk, *fields)
             barrier()
             ksteps, t = timed_leg(L, hk, stream, max(3, args.warmup // 10), max_over_ranks_)
@@ -665,7 +671,8 @@ def run_ours(args):
                 "MLUPS": world * cells * ksteps / t / 1e6, "steps": ksteps, "seconds": t,
                 "bytes_per_cell": kbytes,
                 "hbm_frac": kbytes * cells * ksteps / t / 1e9 / hbm,
-                "note": what + ("fused: one launch per step" if kvec else "moments pass + step")}
+                "note": what + {None: "two steps per pass", 1: "fused: one launch per step",
+                                 0: "moments pass + step"}[kvec]}
         for vp in ("fp64", "ff", "fp32_dev", "fp16_dev"):
             if vp == prec:
                 continue
@@ -673,8 +680,9 @@ def run_ours(args):
             L.lbmhd_init(hv, *fields)
             barrier()
             vsteps, t = timed_leg(L, hv, stream, max(3, args.warmup // 10), max_over_ranks_)
+            # bytes of a step: a pass over the state may take several steps
+            vb = L.lbmhd_bytes_per_cell(vp) * L.lbmhd_launch_count(hv) / L.lbmhd_step_count(hv)
             L.lbmhd_destroy(hv)
-            vb = L.lbmhd_bytes_per_cell(vp)
             variants[vp] = {
                 "MLUPS": world * cells * vsteps / t / 1e6, "steps": vsteps, "seconds": t,
                 "bytes_per_cell": vb,
@@ -816,7 +824,8 @@ def run_ours(args):
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": hbm, "unit": "GB/s",
                          "frac": achieved / hbm, "traffic": traffic,
                          "peak_source": f"{peak_kind} copy bandwidth (MEASURED_PEAKS.json)",
-                         "bytes_per_cell": bpc},
+                         "bytes_per_cell": bpc, "steps_per_pass": args.steps / launches,
+                         "frac_at_one_pass_per_step": bpc * cells * args.steps / dt / 1e9 / hbm},
             "cpu_baseline": cpu, "e2e": e2e, "gpu_launches": int(launches),
             "diagnostics": diagnostics,
             "clocks": clk.summary(), "variants": variants, "variants_3d": variants3d,

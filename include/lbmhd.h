@@ -520,7 +520,11 @@ void lbmhd3_destroy(lbmhd3_t* h);
  * per segment of a column strip of a run; vec 1), or the moments pass and
  * the step over every run's nodes (vec 0, `block` nodes per unit); the batch
  * holds five moment planes per run for the latter.  The default is the
- * single lattice's choice: two-pass for FP64, and for FF with les 2. */
+ * single lattice's choice: two-pass for FP64, and for FF with les 2.
+ * FP32 and FP16 ensembles with les 0 or 1 advance four steps per launch in
+ * one pass over every run where four follow each other and the ensemble is
+ * of a size that gains by it (the same bits; lbmhd_batch_set_launch turns it
+ * off, lbmhd_batch_autotune turns it on again). */
 typedef struct lbmhd_batch_t lbmhd_batch_t;
 
 /* Arrays of nruns entries (caller-owned, not retained).  Every run is
@@ -559,6 +563,7 @@ int lbmhd_batch_get_launch(const lbmhd_batch_t* b, int* vec, int* block, int* st
  * trial_steps steps on a rest state and keeps the fastest.  Results are
  * cached in the JSON file cache_path (key: GPU name, precision, the
  * multiset of lattice shapes); a cached key is applied without timing.
+ * The shape serves the steps that are not taken in passes of four.
  * cache_path may be NULL (no cache).  Must run before any
  * lbmhd_batch_init (ESTATE otherwise); best_mlups (may be NULL) receives
  * the winner's throughput. */

@@ -1,5 +1,10 @@
 // lbmhd_batch.cu -- an ensemble of independent lattices (uneven sizes,
-// own C_S and relaxation times) advanced together by one persistent kernel.
+// own C_S and relaxation times) advanced together by one launch.
+//
+// FP32 and FP16 ensembles with les 0 or 1 that are small or large enough take
+// four steps per pass (batch_pipe_kernel, lbmhd_step_pipe.cu) and the steps
+// that are left over one at a time; the rest of this comment is about the
+// one-step kernel, which also serves every shape that is asked for.
 //
 // All runs live in one pair of buffers (each run a 19-plane block).  The
 // work of one step is cut into units of `block` threads; a unit belongs to

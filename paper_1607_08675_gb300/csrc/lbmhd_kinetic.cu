@@ -11,7 +11,8 @@
 //     (filtered_shift) and collide (collide<..., KIN>) -- or, for les = 3,
 //     the closure's relaxation times (carati_taus) and collide with them.
 // One node per thread; neighbouring threads share the moment loads in L1.
-// The default is a fused one-pass kernel (below) with the same arithmetic.
+// The default is a fused one-pass kernel (below) with the same arithmetic;
+// large FP32 and FP16 lattices take two steps per pass (kin_pipe_kernel).
 // This file is compiled without FMA contraction (-fmad=false), so that the
 // two kernels, whose code is shaped differently, round every operation the
 // same way and give the same bits.

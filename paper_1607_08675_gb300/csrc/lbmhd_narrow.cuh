@@ -8,7 +8,8 @@
 // Initialisation: the equilibria are formed in double-word FP32
 // (lbmhd_ff.cuh) with a bound on their error, and rounded to FP32.  Where
 // the bound leaves the rounding open the node takes the FP64 path, so the
-// stored bits are those of FP64 arithmetic whatever the input.
+// stored values are those of FP64 arithmetic whatever the input (a zero may
+// lose its sign).
 //
 // Measured on GB300 (ms, before -> after): init of 8192^2 FP16 18.55 -> 3.44,
 // 1999 x 1201 FP32 deviations 0.593 -> 0.115, 256^3 FP32 13.34 -> 2.53 (FP32
