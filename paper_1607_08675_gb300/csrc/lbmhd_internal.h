@@ -62,14 +62,16 @@ bool step_variant_ok(int prec, int vec, int nx);
 // format has no such kernel.
 constexpr int kPipeSteps = 4;
 int pipe_steps(int prec, long long nodes, bool kin);
-cudaError_t launch_pipe(int prec, int steps, const void* src, void* dst, const Geom& g,
-                        const HostColl& c, int sm_count, cudaStream_t st);
+cudaError_t launch_pipe(int prec, int steps, int seglen, const void* src, void* dst, const Geom& g,
+                        const HostColl& c, cudaStream_t st);
+// Rows of a warp's segment for such a pass (kin: of two steps of a closure).
+int pipe_seglen(int prec, int steps, int nx, int ny, bool kin, int sm_count);
 
 // Two steps of a kinetic closure (g.kin 2 or 3) in one pass, for the same
 // formats: the bits of two launch_step_kinetic calls.
 constexpr int kKinPipeSteps = 2;
-cudaError_t launch_kin_pipe(int prec, const void* src, void* dst, const Geom& g, const HostColl& c,
-                            int sm_count, cudaStream_t st);
+cudaError_t launch_kin_pipe(int prec, int seglen, const void* src, void* dst, const Geom& g,
+                            const HostColl& c, cudaStream_t st);
 
 // kPipeSteps steps of every run of an ensemble in one pass.  batch_pipe_plan
 // gives the rows of a segment and each run's strips (RunDev::pseglen,
@@ -168,6 +170,7 @@ struct lbmhd_t {
     int vec, block;   // register kernel: nodes per thread, threads per block
     int tma_w;        // > 0: TMA-staged kernel with this tile width
     int pipe;         // most steps of a pass (lbmhd_step_pipe.cu) where steps follow each other, 0: one per launch
+    int pipe_len[lbmhd::kPipeSteps + 1];  // rows of a segment of a pass of 2 .. h->pipe steps
     int kin_two_pass; // les 2, 3: moments pass + step instead of the fused kernel
     int sm_count;
     cudaGraphExec_t graph;

@@ -169,9 +169,9 @@ int next_steps(const lbmhd_t* h, int left) {
 // One launch of k steps from src to dst.
 cudaError_t launch_steps(lbmhd_t* h, int k, const void* src, void* dst) {
     if (k > 1 && h->coll.kin)
-        return launch_kin_pipe(h->p.precision, src, dst, h->geom, h->coll, h->sm_count, h->stream);
+        return launch_kin_pipe(h->p.precision, h->pipe_len[k], src, dst, h->geom, h->coll, h->stream);
     if (k > 1)
-        return launch_pipe(h->p.precision, k, src, dst, h->geom, h->coll, h->sm_count, h->stream);
+        return launch_pipe(h->p.precision, k, h->pipe_len[k], src, dst, h->geom, h->coll, h->stream);
     return launch_one(h, src, dst);
 }
 
@@ -289,7 +289,6 @@ int lbmhd_create(int nx, int ny, const lbmhd_params* p, lbmhd_t** out) {
                : h->vec == 4 || p->precision == LBMHD_FP64 ? 64
                : p->precision == LBMHD_FF && !ff_small ? 256 : 128;
     h->tma_w = 0;
-    h->pipe = pipe_steps(p->precision, (long long)nx * ny, h->coll.kin != 0);
     // Kinetic steps: the fused kernel where it is faster (measured at 8192^2
     // / 4096^2, MLUPS fused vs two-pass: FP32 les 2 33.5K vs 23.7K, les 3
     // 37.1K vs 22.3K; FP16 38.9K vs 26.6K; FF les 3 8.2K vs 7.2K), the
@@ -300,6 +299,9 @@ int lbmhd_create(int nx, int ny, const lbmhd_params* p, lbmhd_t** out) {
             cudaSuccess ||
         h->sm_count < 1)
         h->sm_count = 1;
+    h->pipe = pipe_steps(p->precision, (long long)nx * ny, h->coll.kin != 0);
+    for (int k = 2; k <= h->pipe; ++k)
+        h->pipe_len[k] = pipe_seglen(p->precision, k, nx, ny, h->coll.kin != 0, h->sm_count);
     h->cur = 0;
     *out = h;
     return LBMHD_OK;

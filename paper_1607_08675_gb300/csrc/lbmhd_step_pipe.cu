@@ -39,13 +39,12 @@
 // c_y = 0 planes -- L1 takes what shared memory leaves, and it holds the
 // rows in flight; with the largest shared-memory carve-out S = 2 fell to
 // 57 G, and any spilled register costs half the rate.
-#include <algorithm>
-
 #include "lbmhd_batch_run.cuh"
 #include "lbmhd_cp_async.cuh"
 #include "lbmhd_internal.h"
 #include "lbmhd_pair.cuh"
 #include "lbmhd_pdl.cuh"
+#include "lbmhd_pipe_plan.h"
 #include "lbmhd_step_body.cuh"
 
 namespace lbmhd {
@@ -135,19 +134,6 @@ __host__ __device__ constexpr int keep_slot(int p) {
     return n;
 }
 
-template <int S>
-struct PipeShape {
-    static constexpr int kHalo = (S + 1) / 2 * 2;             // columns left of the output
-    static constexpr int kUseful = (64 - kHalo - S) / 2 * 2;  // output columns of a strip
-};
-
-// Warps per scheduler that the registers are cut for (65536 / 128 / warps).
-// FP32: 128 registers at S = 2, 168 at S = 3, 255 at S = 4 (three warps spill
-// there: 72 G); FP16, whose history is packed, 128 at every S.
-__host__ __device__ constexpr int pipe_warps(int prec, int steps) {
-    return prec == P_FP16_DEV || steps == 2 ? 4 : (steps == 3 ? 3 : 2);
-}
-
 // The populations that stream along y into row r0 of the lane's columns xa, xb
 // (fetched ahead into pre by cp.async, or into z), and on to the next row.
 template <int P, bool AL, int N>
@@ -223,7 +209,7 @@ __device__ __forceinline__ void pipe_body(const typename Fmt<P>::S* __restrict__
                                           const Coll<float>& c, PipeShared<P, S, AL>& sh) {
     using T = typename Fmt<P>::S;
     using Q = typename PairOf<P>::T;
-    constexpr int HL = PipeShape<S>::kHalo, U = PipeShape<S>::kUseful;
+    constexpr int HL = pipe_halo(S), U = pipe_useful(S);
     constexpr bool PF = PipeShared<P, S, AL>::PF;
     auto& pre = sh.pre;
     auto& keep = sh.keep;
@@ -465,7 +451,7 @@ __global__ void __launch_bounds__(32, 4 * kin_pipe_warps(P))
 }
 
 template <int P, int S, bool AL>
-__global__ void __launch_bounds__(32, 4 * pipe_warps(P, S))
+__global__ void __launch_bounds__(32, 4 * pipe_warps(sizeof(typename Fmt<P>::S), S))
     pipe_kernel(const typename Fmt<P>::S* __restrict__ src, typename Fmt<P>::S* __restrict__ dst,
                 int nx, int ny, long long ps, int strips, int seglen, Coll<float> c) {
     __shared__ PipeShared<P, S, AL> sh;
@@ -476,12 +462,9 @@ __global__ void __launch_bounds__(32, 4 * pipe_warps(P, S))
 }
 
 // kPipeSteps steps of every run of an ensemble, a warp per strip-segment of a
-// run, so every run gets the bits of its own lattice.  The run's rates are
-// read by every lane into registers, so FP16 has the registers of three
-// warps per scheduler here, not four.
-constexpr int batch_pipe_warps(int prec) { return prec == P_FP16_DEV ? 3 : 2; }
+// run, so every run gets the bits of its own lattice.
 template <int P, bool AL>
-__global__ void __launch_bounds__(32, 4 * batch_pipe_warps(P))
+__global__ void __launch_bounds__(32, 4 * batch_pipe_warps(sizeof(typename Fmt<P>::S)))
     batch_pipe_kernel(const RunDev<float>* __restrict__ runs, const int* __restrict__ unit_run,
                       const typename Fmt<P>::S* __restrict__ src, typename Fmt<P>::S* __restrict__ dst) {
     __shared__ PipeShared<P, kPipeSteps, AL> sh;
@@ -494,69 +477,33 @@ __global__ void __launch_bounds__(32, 4 * batch_pipe_warps(P))
                                  min(y0 + rd.pseglen, rd.ny), c, sh);
 }
 
-// Rows per segment, at most 96 (longer ones let neighbouring strips drift
-// apart and their shared columns leave L2: 8192^2, S = 4, 96 rows 127.9 G,
-// 192 rows 124 G).  The time of a launch is its rounds of resident warps
-// times the rows a warp walks (its segment, the 2 (S - 1) rows around it and
-// about one for the start) times the time of a row, which grows with the
-// warps w that share a scheduler as a + b w microseconds (measured: S = 4
-// 1.25 at one warp, 2.05 at two; S = 3 2.39 at three).  Within 3% of the best
-// length of a sweep at 1024^2, 1999 x 1201, 2048^2 and 8192^2, where a length
-// that leaves part of a round empty costs up to 60%.
-template <class Units>
-int best_seglen(int S, int warps, int most, int sm_count, Units units_of) {
-    const double a = S == 2 ? 0.8 : (S == 3 ? 0.56 : 0.45), b = S == 2 ? 0.6 : (S == 3 ? 0.61 : 0.8);
-    const double sched = 4.0 * sm_count;
-    const long long resident = 4LL * warps * sm_count;
-    int best = 1;
-    double best_t = 1e300;
-    for (int len = 1; len <= std::min(most, 96); ++len) {
-        const long long units = units_of(len);
-        const long long rounds = units / resident, rest = units % resident;
-        double t = (double)rounds * (a + b * warps);
-        if (rest) t += a + b * (rest > sched ? (double)rest / sched : 1.0);
-        t *= len + 2 * (S - 1) + 1;
-        if (t < best_t) {
-            best_t = t;
-            best = len;
-        }
-    }
-    return best;
-}
-
 template <int P, int S, bool AL>
-cudaError_t launch_pipe_t(const void* src, void* dst, const Geom& g, const HostColl& hc, int sm_count,
+cudaError_t launch_pipe_t(int seglen, const void* src, void* dst, const Geom& g, const HostColl& hc,
                           cudaStream_t st) {
     using T = typename Fmt<P>::S;
-    const int strips = (g.nx + PipeShape<S>::kUseful - 1) / PipeShape<S>::kUseful;
-    const int seglen = best_seglen(S, pipe_warps(P, S), g.ny, sm_count, [&](int len) {
-        return (long long)strips * ((g.ny + len - 1) / len);
-    });
+    const int strips = (g.nx + pipe_useful(S) - 1) / pipe_useful(S);
     const int nseg = (g.ny + seglen - 1) / seglen;
     return launch_after(pipe_kernel<P, S, AL>, (unsigned)strips * (unsigned)nseg, 32, st, (const T*)src,
                         (T*)dst, g.nx, g.ny, g.ps, strips, seglen, coll_for_prec<float>(hc, P));
 }
 
 template <int P>
-cudaError_t launch_pipe_p(int steps, const void* src, void* dst, const Geom& g, const HostColl& c,
-                          int sm_count, cudaStream_t st) {
+cudaError_t launch_pipe_p(int steps, int seglen, const void* src, void* dst, const Geom& g,
+                          const HostColl& c, cudaStream_t st) {
     const bool al = g.nx % 2 == 0;
     switch (steps) {
-        case 2: return (al ? launch_pipe_t<P, 2, true> : launch_pipe_t<P, 2, false>)(src, dst, g, c, sm_count, st);
-        case 3: return (al ? launch_pipe_t<P, 3, true> : launch_pipe_t<P, 3, false>)(src, dst, g, c, sm_count, st);
-        case 4: return (al ? launch_pipe_t<P, 4, true> : launch_pipe_t<P, 4, false>)(src, dst, g, c, sm_count, st);
+        case 2: return (al ? launch_pipe_t<P, 2, true> : launch_pipe_t<P, 2, false>)(seglen, src, dst, g, c, st);
+        case 3: return (al ? launch_pipe_t<P, 3, true> : launch_pipe_t<P, 3, false>)(seglen, src, dst, g, c, st);
+        case 4: return (al ? launch_pipe_t<P, 4, true> : launch_pipe_t<P, 4, false>)(seglen, src, dst, g, c, st);
     }
     return cudaErrorInvalidValue;
 }
 
 template <int P>
-cudaError_t launch_kin_pipe_p(const void* src, void* dst, const Geom& g, const HostColl& hc, int sm_count,
+cudaError_t launch_kin_pipe_p(int seglen, const void* src, void* dst, const Geom& g, const HostColl& hc,
                               cudaStream_t st) {
     using T = typename Fmt<P>::S;
     const int strips = (g.nx + kKinUseful - 1) / kKinUseful;
-    const int seglen = best_seglen(4, kin_pipe_warps(P), g.ny, sm_count, [&](int len) {
-        return (long long)strips * ((g.ny + len - 1) / len);
-    });
     const bool al = g.nx % 2 == 0;
     auto k = hc.kin == 3 ? (al ? kin_pipe_kernel<P, 3, true> : kin_pipe_kernel<P, 3, false>)
                          : (al ? kin_pipe_kernel<P, 2, true> : kin_pipe_kernel<P, 2, false>);
@@ -566,12 +513,12 @@ cudaError_t launch_kin_pipe_p(const void* src, void* dst, const Geom& g, const H
 
 }  // namespace
 
-cudaError_t launch_kin_pipe(int prec, const void* src, void* dst, const Geom& g, const HostColl& c,
-                            int sm_count, cudaStream_t st) {
+cudaError_t launch_kin_pipe(int prec, int seglen, const void* src, void* dst, const Geom& g,
+                            const HostColl& c, cudaStream_t st) {
     switch (prec) {
-        case P_FP32: return launch_kin_pipe_p<P_FP32>(src, dst, g, c, sm_count, st);
-        case P_FP32_DEV: return launch_kin_pipe_p<P_FP32_DEV>(src, dst, g, c, sm_count, st);
-        case P_FP16_DEV: return launch_kin_pipe_p<P_FP16_DEV>(src, dst, g, c, sm_count, st);
+        case P_FP32: return launch_kin_pipe_p<P_FP32>(seglen, src, dst, g, c, st);
+        case P_FP32_DEV: return launch_kin_pipe_p<P_FP32_DEV>(seglen, src, dst, g, c, st);
+        case P_FP16_DEV: return launch_kin_pipe_p<P_FP16_DEV>(seglen, src, dst, g, c, st);
     }
     return cudaErrorInvalidValue;
 }
@@ -583,18 +530,28 @@ int pipe_steps(int prec, long long nodes, bool kin) {
     return large || nodes <= kPipeSmall ? kPipeSteps : 0;
 }
 
+int pipe_seglen(int prec, int steps, int nx, int ny, bool kin, int sm_count) {
+    const int bytes = storage_bytes(prec), useful = kin ? kKinUseful : pipe_useful(steps);
+    const long long strips = (nx + useful - 1) / useful;
+    // a kinetic closure: the rows around a segment and the time of a row are
+    // about those of four steps
+    return pipe_plan(kin ? kPipeSteps : steps, kin ? kin_pipe_warps(prec) : pipe_warps(bytes, steps), ny,
+                     sm_count, [&](int len) { return strips * ((ny + len - 1) / len); })
+        .seglen;
+}
+
 int batch_pipe_plan(int prec, int nruns, const int* nx, const int* ny, int sm_count, int* strips) {
-    constexpr int U = PipeShape<kPipeSteps>::kUseful;
+    constexpr int U = pipe_useful(kPipeSteps);
     int most = 1;
     for (int r = 0; r < nruns; ++r) {
         strips[r] = (nx[r] + U - 1) / U;
         most = std::max(most, ny[r]);
     }
-    return best_seglen(kPipeSteps, batch_pipe_warps(prec), most, sm_count, [&](int len) {
+    return pipe_plan(kPipeSteps, batch_pipe_warps(storage_bytes(prec)), most, sm_count, [&](int len) {
         long long u = 0;
         for (int r = 0; r < nruns; ++r) u += (long long)strips[r] * ((ny[r] + len - 1) / len);
         return u;
-    });
+    }).seglen;
 }
 
 cudaError_t launch_batch_pipe(int prec, bool even, const void* runs, const int* unit_run,
@@ -613,12 +570,12 @@ cudaError_t launch_batch_pipe(int prec, bool even, const void* runs, const int* 
     return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_pipe(int prec, int steps, const void* src, void* dst, const Geom& g,
-                        const HostColl& c, int sm_count, cudaStream_t st) {
+cudaError_t launch_pipe(int prec, int steps, int seglen, const void* src, void* dst, const Geom& g,
+                        const HostColl& c, cudaStream_t st) {
     switch (prec) {
-        case P_FP32: return launch_pipe_p<P_FP32>(steps, src, dst, g, c, sm_count, st);
-        case P_FP32_DEV: return launch_pipe_p<P_FP32_DEV>(steps, src, dst, g, c, sm_count, st);
-        case P_FP16_DEV: return launch_pipe_p<P_FP16_DEV>(steps, src, dst, g, c, sm_count, st);
+        case P_FP32: return launch_pipe_p<P_FP32>(steps, seglen, src, dst, g, c, st);
+        case P_FP32_DEV: return launch_pipe_p<P_FP32_DEV>(steps, seglen, src, dst, g, c, st);
+        case P_FP16_DEV: return launch_pipe_p<P_FP16_DEV>(steps, seglen, src, dst, g, c, st);
     }
     return cudaErrorInvalidValue;
 }
