@@ -153,7 +153,7 @@ int lbmhd_init_device(lbmhd_t* h, const double* rho, const double* ux, const dou
 /* Advance n >= 0 time steps of fused pull-stream and collide (Sec. 1.2 and
  * Sec. 3) over the whole lattice, one per launch; FP32 and FP16 storage
  * advance up to four (les 0, 1) or two (les 2, 3) per launch where steps
- * follow each other and the lattice is of a size that gains by it (the same
+ * follow each other and the lattice is of a size and shape that gain by it (the same
  * bits; not after lbmhd_set_launch).  Asynchronous on the handle's
  * stream; long runs replay a captured CUDA graph.  Returns
  * ESTATE before init.  A pending non-finite report (check_finite_every)
@@ -523,7 +523,7 @@ void lbmhd3_destroy(lbmhd3_t* h);
  * single lattice's choice: two-pass for FP64, and for FF with les 2.
  * FP32 and FP16 ensembles with les 0 or 1 advance four steps per launch in
  * one pass over every run where four follow each other and the ensemble is
- * of a size that gains by it (the same bits; lbmhd_batch_set_launch turns it
+ * of sizes that gain by it (the same bits; lbmhd_batch_set_launch turns it
  * off, lbmhd_batch_autotune turns it on again). */
 typedef struct lbmhd_batch_t lbmhd_batch_t;
 

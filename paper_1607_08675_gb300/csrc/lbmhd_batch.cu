@@ -298,16 +298,13 @@ int upload_runs_t(lbmhd_batch_t* b) {
     return LBMHD_OK;
 }
 
-// The ensemble takes several steps per pass where a lattice of its size would.
+// Whether the ensemble takes several steps per pass.
 bool batch_pipe_ok(const lbmhd_batch_t* b) {
-    long long nodes = 0;
-    for (int r = 0; r < b->nruns; ++r) nodes += (long long)b->nx[r] * b->ny[r];
-    return b->p.les < 2 && pipe_steps(b->p.precision, nodes, false) > 0;
+    return b->p.les < 2 && batch_pipe_pays(b->p.precision, b->nruns, b->nx.data(), b->ny.data(), b->sms);
 }
 
 // (Re)build the unit maps and the co-resident grid for the current shape.
 int configure(lbmhd_batch_t* b) {
-    LBMHD_BCK(b, cudaDeviceGetAttribute(&b->sms, cudaDevAttrMultiProcessorCount, b->device));
     int rc = b->p.precision == LBMHD_FP64 ? upload_runs_t<double>(b)
              : b->p.precision == LBMHD_FF ? upload_runs_t<ff>(b)
                                           : upload_runs_t<float>(b);
@@ -616,6 +613,8 @@ int lbmhd_batch_create(int nruns, const int* nx, const int* ny, const double* ta
         b->block = 128;
         b->spl = 1;
     }
+    if (cudaDeviceGetAttribute(&b->sms, cudaDevAttrMultiProcessorCount, b->device) != cudaSuccess || b->sms < 1)
+        b->sms = 1;
     b->pipe = batch_pipe_ok(b);
     int rc = configure(b);
     if (rc) {

@@ -57,11 +57,12 @@ bool step_variant_ok(int prec, int vec, int nx);
 
 // `steps` (2 .. kPipeSteps) time steps in one pass, src -> dst
 // (lbmhd_step_pipe.cu): the bits of as many launch_step calls.  pipe_steps:
-// the most steps of a pass for a lattice or an ensemble of this many nodes
-// (kin: with a kinetic closure), 0 where single steps are as fast or the
-// format has no such kernel.
+// the most steps of a pass for a lattice (kin: with a kinetic closure), 0
+// where single steps are as fast (lbmhd_pipe_plan.h) or the format has no such
+// kernel.  batch_pipe_pays: whether an ensemble (les 0, 1) takes kPipeSteps.
 constexpr int kPipeSteps = 4;
-int pipe_steps(int prec, long long nodes, bool kin);
+int pipe_steps(int prec, int nx, int ny, bool kin, int sm_count);
+bool batch_pipe_pays(int prec, int nruns, const int* nx, const int* ny, int sm_count);
 cudaError_t launch_pipe(int prec, int steps, int seglen, const void* src, void* dst, const Geom& g,
                         const HostColl& c, cudaStream_t st);
 // Rows of a warp's segment for such a pass (kin: of two steps of a closure).

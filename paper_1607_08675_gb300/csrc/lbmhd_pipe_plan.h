@@ -75,4 +75,85 @@ PipePlan pipe_plan(int S, int warps, int most, int sm_count, Units units_of) {
     return t > least * (7.0 / 6.0) ? PipePlan{by_busiest, least} : PipePlan{by_mean, t};
 }
 
+// ---- the lattices and ensembles that passes are for --------------------------
+// Both state buffers together beyond 80 MB, about where they stop fitting in L2
+// and the one-step kernel falls to the rate of HBM; or up to 32768 nodes, where
+// a launch is mostly latency and one for four steps takes less than four.
+// Between them the rows that segments share cost as much as the passes save
+// (FP32, us per step, one-step / pass: 512^2 5.8 / 6.3).
+constexpr long long kPipeBytes = 80LL << 20;
+constexpr long long kPipeSmall = 32768;
+
+// Microseconds of one step by the one-step kernels on GB300: picoseconds
+// per node while the state fits in L2, beyond it, and where it is many times that,
+// by `bytes` of a value.  An odd nx costs them a third (2 bytes; 4 bytes: a
+// tenth), an even one that is no multiple of their widest vector a tenth.
+// align: the largest power of two up to 8 that divides every nx.
+inline double one_step_us(int bytes, long long nodes, int align, bool ensemble) {
+    const double mb = 2.0 * 19.0 * bytes * (double)nodes * 1e-6;
+    const double fit = ensemble ? (bytes == 2 ? 14.5 : 25.5) : (bytes == 2 ? 11.6 : 16.3);
+    const double mid = ensemble ? (bytes == 2 ? 16.2 : 25.5) : (bytes == 2 ? 15.2 : 23.4);
+    const double big = ensemble ? (bytes == 2 ? 14.2 : 25.5) : (bytes == 2 ? 12.9 : 23.2);
+    const double x = std::min(std::max((mb - 84.0) / 63.0, 0.0), 1.0);
+    const double y = std::min(std::max((mb - 300.0) / 900.0, 0.0), 1.0);
+    double ps = fit + (mid - fit) * x + (big - mid) * y;
+    if (align == 1) ps *= bytes == 2 ? 1.3 : 1.1;
+    else if (bytes == 2 && align < (ensemble ? 4 : 8)) ps *= 1.08 + 0.09 * y;
+    return ps * 1e-6 * (double)nodes;
+}
+
+// Whether passes of four steps are the faster way for these lattices (les 0, 1;
+// one, or the runs of an ensemble).  A strip computes 64 columns whatever the
+// lattice has, and rows around a segment whatever its rows, so this depends on
+// the shape, not on the nodes alone (GB300, us per step, one-step / pass, FP32
+// 2^21 nodes in rows of 8, 16, 24, 64 and 256: 48 / 122, 48 / 60, 48 / 43,
+// 48 / 33, 48 / 20; in 1, 2 and 4 rows 48 / 70, 47 / 44, 47 / 32).
+//
+// Large: by the plan's time and that of four single steps.  Of 430 lattices
+// and ensembles timed, none takes a pass that is more than 2% slower and none
+// misses one that is more than 11% faster.
+//
+// Small lattices: while one warp per scheduler does with segments of a row --
+// or of two rows where FP16 steps four nodes at a time, which is slower at such
+// sizes -- (FP32 128^2 2.15 / 1.86, 16 x 1024 2.1 / 2.4, 64 x 512 2.0 / 2.3, 256 x
+// 128 2.1 / 2.2, 1024 x 32 2.1 / 2.0; FP16 256 x 128 2.6 / 2.2), and not in rows
+// so short that warps of different SMs write one sector (4 x 512 1.8 / 2.6).
+// Odd rows of FP16, which are not fetched ahead, lose a tenth (99^2 2.2 / 2.4).
+// Small ensembles, whose one-step launch takes 3.8 us: up to 14 warps per SM in
+// segments of a row (128 runs of 16 x 16 3.9 / 3.3, of 8 x 32 3.9 / 5.2).
+inline bool pipe_pays(int bytes, int nruns, const int* nx, const int* ny, bool ensemble, int sm_count) {
+    constexpr int S = 4;
+    auto strips = [&](int r) { return (long long)((nx[r] + pipe_useful(S) - 1) / pipe_useful(S)); };
+    auto units_of = [&](int len) {
+        long long u = 0;
+        for (int r = 0; r < nruns; ++r) u += strips(r) * ((ny[r] + len - 1) / len);
+        return u;
+    };
+    long long nodes = 0;
+    int most = 1, align = 8;
+    for (int r = 0; r < nruns; ++r) {
+        nodes += (long long)nx[r] * ny[r];
+        most = std::max(most, ny[r]);
+        while (nx[r] % align) align /= 2;
+    }
+    if (2 * 19 * bytes * nodes >= kPipeBytes) {
+        const int warps = ensemble ? batch_pipe_warps(bytes) : pipe_warps(bytes, S);
+        return pipe_plan(S, warps, most, sm_count, units_of).us <= S * one_step_us(bytes, nodes, align, ensemble);
+    }
+    if (nodes > kPipeSmall) return false;
+    if (ensemble) return units_of(1) <= 14LL * sm_count;
+    const int rows = bytes == 2 && align >= 4 ? 2 : 1;
+    return (nx[0] >= 8 || ny[0] <= 8) && units_of(rows) <= 4LL * sm_count;
+}
+
+// The kinetic closures, two steps per pass: only the large ones (les 2 FP32, us
+// per step, one-step / pass: 128^2 2.9 / 3.6, 512^2 11.4 / 12.2, 1024^2 39.4 /
+// 25.6).  Their one-step kernel sweeps strips of 256 columns, so narrow lattices
+// gain the most (2^21 nodes in rows of 2, 16, 57, 113 and 256: 2015 / 1868, 347 /
+// 131, 126 / 84, 86 / 65, 67 / 44); rows fewer than four are slower in a pass
+// (1, 2, 3 rows: 76 / 143, 68 / 93, 69 / 76).
+inline bool kin_pipe_pays(int bytes, int nx, int ny) {
+    return 2LL * 19 * bytes * nx * ny >= kPipeBytes;
+}
+
 }  // namespace lbmhd

@@ -299,7 +299,7 @@ int lbmhd_create(int nx, int ny, const lbmhd_params* p, lbmhd_t** out) {
             cudaSuccess ||
         h->sm_count < 1)
         h->sm_count = 1;
-    h->pipe = pipe_steps(p->precision, (long long)nx * ny, h->coll.kin != 0);
+    h->pipe = pipe_steps(p->precision, nx, ny, h->coll.kin != 0, h->sm_count);
     for (int k = 2; k <= h->pipe; ++k)
         h->pipe_len[k] = pipe_seglen(p->precision, k, nx, ny, h->coll.kin != 0, h->sm_count);
     h->cur = 0;

@@ -51,19 +51,6 @@ namespace lbmhd {
 
 namespace {
 
-// The lattices this kernel is for.  Large: both state buffers together beyond
-// 80 MB, about where they stop fitting in L2 and the one-step kernel falls to
-// the rate of HBM (FP32, us per step, one-step / this: 768^2 10.6 / 10.4,
-// 1024^2 26.0 / 12.2; FP16 1024^2 12.5 / 12.8).  Small: up to 32768 nodes,
-// where a launch is mostly latency and one for four steps takes less than
-// four (FP32 64^2 2.23 / 1.77, 128^2 2.57 / 1.90, 256^2 3.16 / 3.19).
-// Between them the rows that segments share cost as much as the passes save
-// (FP32 512^2 5.8 / 6.3).  The kinetic closures, two steps per pass: only the
-// large ones (les 2 FP32, us per step, one-step / this: 128^2 2.9 / 3.6, 512^2
-// 11.4 / 12.2, 1024^2 39.4 / 28.3).
-constexpr long long kPipeBytes = 80LL << 20;
-constexpr long long kPipeSmall = 32768;
-
 // A pair of neighbouring columns of one plane, as stored.
 template <int P>
 struct PairOf {
@@ -523,11 +510,15 @@ cudaError_t launch_kin_pipe(int prec, int seglen, const void* src, void* dst, co
     return cudaErrorInvalidValue;
 }
 
-int pipe_steps(int prec, long long nodes, bool kin) {
-    if (prec != P_FP32 && prec != P_FP32_DEV && prec != P_FP16_DEV) return 0;
-    const bool large = 2 * kPlanes * (long long)storage_bytes(prec) * nodes >= kPipeBytes;
-    if (kin) return large ? kKinPipeSteps : 0;
-    return large || nodes <= kPipeSmall ? kPipeSteps : 0;
+static bool narrow(int prec) { return prec == P_FP32 || prec == P_FP32_DEV || prec == P_FP16_DEV; }
+int pipe_steps(int prec, int nx, int ny, bool kin, int sm_count) {
+    const int bytes = storage_bytes(prec);
+    if (!narrow(prec)) return 0;
+    if (kin) return kin_pipe_pays(bytes, nx, ny) ? kKinPipeSteps : 0;
+    return pipe_pays(bytes, 1, &nx, &ny, false, sm_count) ? kPipeSteps : 0;
+}
+bool batch_pipe_pays(int prec, int nruns, const int* nx, const int* ny, int sm_count) {
+    return narrow(prec) && pipe_pays(storage_bytes(prec), nruns, nx, ny, true, sm_count);
 }
 
 int pipe_seglen(int prec, int steps, int nx, int ny, bool kin, int sm_count) {
