@@ -136,6 +136,7 @@ struct lbmhd_batch_t {
     bool peven;         // every nx is even
     unsigned pnunits;
     int* d_punit_run;
+    RunPass* d_pass;
     unsigned* d_bar;
     int* d_flag;
     int vec, block, spl, grid, sms;
@@ -241,6 +242,7 @@ int kin_seglen(int ny) {
 template <class R>
 int upload_runs_t(lbmhd_batch_t* b) {
     std::vector<RunDev<R>> rd(b->nruns);
+    std::vector<RunPass> pass(b->nruns);
     std::vector<int> map, pmap, pstrips(b->nruns);
     unsigned unit = 0;
     const int pseglen =
@@ -264,9 +266,7 @@ int upload_runs_t(lbmhd_batch_t* b) {
         rd[r].kstrips = (b->nx[r] + ksw - 1) / ksw;
         rd[r].kseglen = kin_seglen(b->ny[r]);
         rd[r].c = coll_for_prec<R>(hc, b->p.precision);
-        rd[r].punit0 = (unsigned)pmap.size();
-        rd[r].pstrips = pstrips[r];
-        rd[r].pseglen = pseglen;
+        pass[r] = {(unsigned)pmap.size(), pstrips[r], pseglen};
         b->peven = b->peven && b->nx[r] % 2 == 0;
         if (b->pipe) pmap.insert(pmap.end(), (size_t)pstrips[r] * ((b->ny[r] + pseglen - 1) / pseglen), r);
         const unsigned units =
@@ -280,14 +280,18 @@ int upload_runs_t(lbmhd_batch_t* b) {
     if (b->d_runs) cudaFree(b->d_runs);
     if (b->d_unit_run) cudaFree(b->d_unit_run);
     if (b->d_punit_run) cudaFree(b->d_punit_run);
+    if (b->d_pass) cudaFree(b->d_pass);
     b->d_runs = nullptr;
     b->d_unit_run = nullptr;
     b->d_punit_run = nullptr;
+    b->d_pass = nullptr;
     b->pnunits = (unsigned)pmap.size();
     if (b->pnunits) {
         LBMHD_BCK(b, cudaMalloc((void**)&b->d_punit_run, pmap.size() * sizeof(int)));
         LBMHD_BCK(b, cudaMemcpy(b->d_punit_run, pmap.data(), pmap.size() * sizeof(int),
                                 cudaMemcpyHostToDevice));
+        LBMHD_BCK(b, cudaMalloc((void**)&b->d_pass, pass.size() * sizeof(RunPass)));
+        LBMHD_BCK(b, cudaMemcpy(b->d_pass, pass.data(), pass.size() * sizeof(RunPass), cudaMemcpyHostToDevice));
     }
     LBMHD_BCK(b, cudaMalloc(&b->d_runs, rd.size() * sizeof(RunDev<R>)));
     LBMHD_BCK(b, cudaMalloc((void**)&b->d_unit_run, map.size() * sizeof(int)));
@@ -373,7 +377,7 @@ cudaError_t launch_batch(lbmhd_batch_t* b, int nsteps, int parity) {
 // to be dropped (there is no barrier in it).
 bool use_pipe(const lbmhd_batch_t* b) { return b->pipe && b->pnunits && !b->drop_arrival; }
 cudaError_t launch_pass(lbmhd_batch_t* b, int parity) {
-    return launch_batch_pipe(b->p.precision, b->peven, b->d_runs, b->d_punit_run, b->pnunits,
+    return launch_batch_pipe(b->p.precision, b->peven, b->d_runs, b->d_pass, b->d_punit_run, b->pnunits,
                              b->buf[parity & 1], b->buf[1 - (parity & 1)], b->stream);
 }
 
@@ -917,6 +921,7 @@ void lbmhd_batch_destroy(lbmhd_batch_t* b) {
     cudaFree(b->d_runs);
     cudaFree(b->d_unit_run);
     cudaFree(b->d_punit_run);
+    cudaFree(b->d_pass);
     cudaFree(b->d_mom);
     cudaFree(b->d_bar);
     cudaFree(b->d_flag);

@@ -75,10 +75,11 @@ cudaError_t launch_kin_pipe(int prec, int seglen, const void* src, void* dst, co
                             const HostColl& c, cudaStream_t st);
 
 // kPipeSteps steps of every run of an ensemble in one pass.  batch_pipe_plan
-// gives the rows of a segment and each run's strips (RunDev::pseglen,
-// pstrips, units = strips x segments); even: every run's nx is even.
+// gives the rows of a segment and each run's strips (units = strips x
+// segments); even: every run's nx is even.
+struct RunPass;
 int batch_pipe_plan(int prec, int nruns, const int* nx, const int* ny, int sm_count, int* strips);
-cudaError_t launch_batch_pipe(int prec, bool even, const void* runs, const int* unit_run,
+cudaError_t launch_batch_pipe(int prec, bool even, const void* runs, const RunPass* pass, const int* unit_run,
                               unsigned nunits, const void* src, void* dst, cudaStream_t st);
 
 // TMA-staged step (lbmhd_step_tma.cu): W threads = nodes per row tile,

@@ -265,12 +265,14 @@ __host__ __device__ inline Coll<R> make_coll_t(double tn, double te, double k18,
     c.s6 = (R)s6;
     c.s7 = (R)s7;
     c.s8 = (R)s8;
-    c.c5 = (R)(s5 / 12.0);
-    c.c6 = (R)(s6 / 12.0);
-    c.c7 = (R)(s7 / 45.0);
-    c.c8 = (R)(s8 / 20.0);
-    c.fix7 = s7 > 0.0;
-    c.fix8 = s8 > 0.0;
+    if constexpr (std::is_same<R, double>::value) {
+        c.c5 = s5 / 12.0;
+        c.c6 = s6 / 12.0;
+        c.c7 = s7 / 45.0;
+        c.c8 = s8 / 20.0;
+        c.fix7 = s7 > 0.0;
+        c.fix8 = s8 > 0.0;
+    }
     c.les = les;
     c.tie5 = tie5;
     c.tie6 = tie6;

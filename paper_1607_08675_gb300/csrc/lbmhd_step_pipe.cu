@@ -452,16 +452,19 @@ __global__ void __launch_bounds__(32, 4 * pipe_warps(sizeof(typename Fmt<P>::S),
 // run, so every run gets the bits of its own lattice.
 template <int P, bool AL>
 __global__ void __launch_bounds__(32, 4 * batch_pipe_warps(sizeof(typename Fmt<P>::S)))
-    batch_pipe_kernel(const RunDev<float>* __restrict__ runs, const int* __restrict__ unit_run,
-                      const typename Fmt<P>::S* __restrict__ src, typename Fmt<P>::S* __restrict__ dst) {
+    batch_pipe_kernel(const RunDev<float>* __restrict__ runs, const RunPass* __restrict__ pass,
+                      const int* __restrict__ unit_run, const typename Fmt<P>::S* __restrict__ src,
+                      typename Fmt<P>::S* __restrict__ dst) {
     __shared__ PipeShared<P, kPipeSteps, AL> sh;
     after_previous();
-    const RunDev<float>& rd = runs[unit_run[blockIdx.x]];
-    const int l = (int)(blockIdx.x - rd.punit0);
-    const int strip = l % rd.pstrips, y0 = l / rd.pstrips * rd.pseglen;
+    const int r = unit_run[blockIdx.x];
+    const RunDev<float>& rd = runs[r];
+    const RunPass rp = pass[r];
+    const int l = (int)(blockIdx.x - rp.unit0);
+    const int strip = l % rp.strips, y0 = l / rp.strips * rp.seglen;
     const Coll<float> c = rd.c;
     pipe_body<P, kPipeSteps, AL>(src + rd.off, dst + rd.off, rd.nx, rd.ny, rd.ps, strip, y0,
-                                 min(y0 + rd.pseglen, rd.ny), c, sh);
+                                 min(y0 + rp.seglen, rd.ny), c, sh);
 }
 
 template <int P, int S, bool AL>
@@ -545,13 +548,13 @@ int batch_pipe_plan(int prec, int nruns, const int* nx, const int* ny, int sm_co
     }).seglen;
 }
 
-cudaError_t launch_batch_pipe(int prec, bool even, const void* runs, const int* unit_run,
+cudaError_t launch_batch_pipe(int prec, bool even, const void* runs, const RunPass* pass, const int* unit_run,
                               unsigned nunits, const void* src, void* dst, cudaStream_t st) {
     const RunDev<float>* rd = (const RunDev<float>*)runs;
 #define LBMHD_BP(P)                                                                           \
     case P:                                                                                   \
         return launch_after(even ? batch_pipe_kernel<P, true> : batch_pipe_kernel<P, false>, nunits, \
-                            32, st, rd, unit_run, (const Fmt<P>::S*)src, (Fmt<P>::S*)dst);
+                            32, st, rd, pass, unit_run, (const Fmt<P>::S*)src, (Fmt<P>::S*)dst);
     switch (prec) {
         LBMHD_BP(P_FP32)
         LBMHD_BP(P_FP32_DEV)
