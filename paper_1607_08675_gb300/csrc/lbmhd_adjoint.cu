@@ -257,9 +257,9 @@ __device__ __forceinline__ double warp_sum_d(double v) {
 // the blocks follows the sweep.
 template <int P>
 __global__ void __launch_bounds__(kAdjBlock) adj_step_kernel(
-    const typename Fmt<P>::S* __restrict__ x, const typename Fmt<P>::R* __restrict__ lin,
-    typename Fmt<P>::R* __restrict__ lout, int nx, int ny, long long ps,
-    Coll<typename Fmt<P>::R> c, float inv_scale, double* __restrict__ partials) {
+    const typename Fmt<P>::S* x, const typename Fmt<P>::R* lin,
+    typename Fmt<P>::R* lout, int nx, int ny, long long ps,
+    Coll<typename Fmt<P>::R> c, float inv_scale, double* partials) {
     using R = typename Fmt<P>::R;
     after_previous();
     const long long n = (long long)nx * ny;

@@ -12,8 +12,8 @@
 namespace lbmhd {
 
 template <int P, int V>
-__global__ void __launch_bounds__(256) step_kernel(const typename Fmt<P>::S* __restrict__ src,
-                                                   typename Fmt<P>::S* __restrict__ dst, int nx,
+__global__ void __launch_bounds__(256) step_kernel(const typename Fmt<P>::S* src,
+                                                   typename Fmt<P>::S* dst, int nx,
                                                    int ny, long long ps, unsigned total,
                                                    unsigned total_pad,
                                                    Coll<typename Fmt<P>::R> c, float scale,
@@ -27,7 +27,7 @@ __global__ void __launch_bounds__(256) step_kernel(const typename Fmt<P>::S* __r
 // Eight FP16 nodes per thread, held to 128 registers, 16 warps per SM (left to
 // itself ptxas takes 143, 12 warps: 8192^2 933 us per step).
 __global__ void __launch_bounds__(256, 2)
-    step_kernel_h8(const unsigned short* __restrict__ src, unsigned short* __restrict__ dst, int nx,
+    step_kernel_h8(const unsigned short* src, unsigned short* dst, int nx,
                    int ny, long long ps, unsigned total, unsigned total_pad, Coll<float> c,
                    float scale, float inv_scale, int y0) {
     after_previous();

@@ -348,7 +348,7 @@ __device__ __forceinline__ void kin_collide(typename PairOf<P>::T (&z)[kPlanes],
 constexpr int kin_pipe_warps(int prec) { return prec == P_FP16_DEV ? 3 : 2; }
 template <int P, int MODE, bool AL>
 __global__ void __launch_bounds__(32, 4 * kin_pipe_warps(P))
-    kin_pipe_kernel(const typename Fmt<P>::S* __restrict__ src, typename Fmt<P>::S* __restrict__ dst,
+    kin_pipe_kernel(const typename Fmt<P>::S* src, typename Fmt<P>::S* dst,
                     int nx, int ny, long long ps, int strips, int seglen, Coll<float> c) {
     using T = typename Fmt<P>::S;
     using Q = typename PairOf<P>::T;
@@ -439,7 +439,7 @@ __global__ void __launch_bounds__(32, 4 * kin_pipe_warps(P))
 
 template <int P, int S, bool AL>
 __global__ void __launch_bounds__(32, 4 * pipe_warps(sizeof(typename Fmt<P>::S), S))
-    pipe_kernel(const typename Fmt<P>::S* __restrict__ src, typename Fmt<P>::S* __restrict__ dst,
+    pipe_kernel(const typename Fmt<P>::S* src, typename Fmt<P>::S* dst,
                 int nx, int ny, long long ps, int strips, int seglen, Coll<float> c) {
     __shared__ PipeShared<P, S, AL> sh;
     after_previous();
@@ -452,9 +452,9 @@ __global__ void __launch_bounds__(32, 4 * pipe_warps(sizeof(typename Fmt<P>::S),
 // run, so every run gets the bits of its own lattice.
 template <int P, bool AL>
 __global__ void __launch_bounds__(32, 4 * batch_pipe_warps(sizeof(typename Fmt<P>::S)))
-    batch_pipe_kernel(const RunDev<float>* __restrict__ runs, const RunPass* __restrict__ pass,
-                      const int* __restrict__ unit_run, const typename Fmt<P>::S* __restrict__ src,
-                      typename Fmt<P>::S* __restrict__ dst) {
+    batch_pipe_kernel(const RunDev<float>* runs, const RunPass* pass,
+                      const int* unit_run, const typename Fmt<P>::S* src,
+                      typename Fmt<P>::S* dst) {
     __shared__ PipeShared<P, kPipeSteps, AL> sh;
     after_previous();
     const int r = unit_run[blockIdx.x];
