@@ -78,10 +78,11 @@ __device__ __forceinline__ double widen_f32(float v, bool& odd) {
     return __hiloint2double((int)((b & 0x80000000u) | h), (int)(b << 29));
 }
 
-// n[i] / d for i < N with one reciprocal: FP32 seed, one Newton-Raphson step
-// in FP64, and the quotient corrected by its exact remainder (Markstein), two
-// multiply-adds after the product.  The IEEE quotient but for an occasional
-// last place; divisors beyond FP32 range take the division.
+// n[i] / d for i < N (finite n) with one reciprocal: FP32 seed, one step of
+// third order in FP64, and the quotient corrected by its exact remainder
+// (Markstein), two multiply-adds after the product.  Within 0.501 units of the
+// last place, so the IEEE quotient but for an occasional last place (a zero may
+// lose its sign); divisors beyond 2^-60 to 2^60 take the division.
 template <int N>
 __device__ __forceinline__ void divide_all(const double (&n)[N], double d, double (&q)[N]) {
     const unsigned h = (unsigned)__double2hiint(d);
