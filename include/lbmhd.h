@@ -153,9 +153,9 @@ int lbmhd_init_device(lbmhd_t* h, const double* rho, const double* ux, const dou
 /* Advance n >= 0 time steps of fused pull-stream and collide (Sec. 1.2 and
  * Sec. 3) over the whole lattice, one per launch; FP32 and FP16 storage
  * advance up to four (les 0, 1) or two (les 2, 3) per launch where steps
- * follow each other and the lattice is of a size and shape that gain by it (the same
- * bits; not after lbmhd_set_launch).  Asynchronous on the handle's
- * stream; long runs replay a captured CUDA graph.  Returns
+ * follow each other and the lattice is of a size and shape that gain by it
+ * (the same values; not after lbmhd_set_launch).  Asynchronous on the
+ * handle's stream; long runs replay a captured CUDA graph.  Returns
  * ESTATE before init.  A pending non-finite report (check_finite_every)
  * is returned by the next synchronising call. */
 int lbmhd_step(lbmhd_t* h, int n);
@@ -276,11 +276,13 @@ int64_t lbmhd_launch_count(const lbmhd_t* h);
  * available for FP16 storage (16-byte loads).  Default: the register
  * kernel with 2 nodes per thread in 128-thread blocks (FP32 storage), 8
  * nodes in 32-thread blocks (FP16 storage; 4 in 64-thread blocks below 2^20
- * nodes), 1 node in 64-thread blocks (FP64) or 2 nodes in 256-thread blocks (FF; 1 in 128-thread blocks up to
- * 2^18 nodes), falling back to narrower vectors when nx is not a multiple.
- * Results do not depend on the shape (bit for bit).  EINVAL if the shape
- * is not available.  A shape that was set is used for every step; without
- * one, lbmhd_step takes several steps per launch where it can.
+ * nodes), 1 node in 64-thread blocks (FP64) or 2 nodes in 256-thread blocks
+ * (FF; 1 in 128-thread blocks up to 2^18 nodes), falling back to narrower
+ * vectors when nx is not a multiple.  Results do not depend on the shape: bit
+ * for bit but for the sign of a zero, where a state holds negative zeros
+ * (FP32_DEV, FP16_DEV).  EINVAL if the shape is not available.  A shape that
+ * was set is used for every step, also the one that lbmhd_get_launch reports;
+ * without one, lbmhd_step takes several steps per launch where that is faster.
  * For les 2 and 3 (steps that need moment gradients): vec = 1 selects the
  * fused kernel (one launch per step; CTAs sweep column strips; `block`
  * ignored on input, reported as strip width + 32), vec = 0 the two-pass
@@ -523,7 +525,7 @@ void lbmhd3_destroy(lbmhd3_t* h);
  * single lattice's choice: two-pass for FP64, and for FF with les 2.
  * FP32 and FP16 ensembles with les 0 or 1 advance four steps per launch in
  * one pass over every run where four follow each other and the ensemble is
- * of sizes that gain by it (the same bits; lbmhd_batch_set_launch turns it
+ * of sizes that gain by it (the same values; lbmhd_batch_set_launch turns it
  * off, lbmhd_batch_autotune turns it on again). */
 typedef struct lbmhd_batch_t lbmhd_batch_t;
 

@@ -96,7 +96,7 @@ __device__ __forceinline__ R ldg_r(const R* p) {
 }
 
 // Two nodes in one arithmetic type: packed two-wide FP32 (lbmhd_pair.cuh),
-// each operation rounded on its own, so a node gets the bits of the scalar
+// each operation rounded on its own, so a node gets the values of the scalar
 // form.
 struct f2 {
     float2 v;

@@ -56,7 +56,7 @@ cudaError_t launch_step(int prec, int vec, int block, int max_blocks, const void
 bool step_variant_ok(int prec, int vec, int nx);
 
 // `steps` (2 .. kPipeSteps) time steps in one pass, src -> dst
-// (lbmhd_step_pipe.cu): the bits of as many launch_step calls.  pipe_steps:
+// (lbmhd_step_pipe.cu): the values of as many launch_step calls.  pipe_steps:
 // the most steps of a pass for a lattice (kin: with a kinetic closure), 0
 // where single steps are as fast (lbmhd_pipe_plan.h) or the format has no such
 // kernel.  batch_pipe_pays: whether an ensemble (les 0, 1) takes kPipeSteps.
@@ -69,7 +69,7 @@ cudaError_t launch_pipe(int prec, int steps, int seglen, const void* src, void* 
 int pipe_seglen(int prec, int steps, int nx, int ny, bool kin, int sm_count);
 
 // Two steps of a kinetic closure (g.kin 2 or 3) in one pass, for the same
-// formats: the bits of two launch_step_kinetic calls.
+// formats: the values of two launch_step_kinetic calls.
 constexpr int kKinPipeSteps = 2;
 cudaError_t launch_kin_pipe(int prec, int seglen, const void* src, void* dst, const Geom& g,
                             const HostColl& c, cudaStream_t st);

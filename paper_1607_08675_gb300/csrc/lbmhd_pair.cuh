@@ -4,7 +4,8 @@
 // slot for two operations.
 //
 // Both come from the one source below, and every FP32 step kernel calls it, so
-// they give the same bits whatever shape the compiler gives their code.  The
+// they give the same values whatever shape the compiler gives their code, bit
+// for bit but for the sign of a zero (see mul_).  The
 // operations are those of collide() (lbmhd_device.cuh) with its products fused
 // into the sums that follow.  ABS: FP32 storage of the populations themselves
 // fuses the second product of j_x j_y / rho - B_x B_y instead of the first.  A
@@ -31,9 +32,13 @@ __device__ __forceinline__ float fma_(float a, float b, float c) { return __fmaf
 __device__ __forceinline__ float neg_(float a) { return -a; }
 __device__ __forceinline__ float abs_(float a) { return fabsf(a); }
 __device__ __forceinline__ float2 add_(float2 a, float2 b) { return __fadd2_rn(a, b); }
-// A product as a multiply-add of +0 (a zero product may lose its sign, no value
-// changes): ptxas fuses a packed product into a packed sum that follows, with
-// their roundings written out and contraction off, but not a multiply-add.
+// A product as a multiply-add of +0: ptxas fuses a packed product into a packed
+// sum that follows, with their roundings written out and contraction off, but
+// not a multiply-add.  A product that is -0 comes out as +0, which only a sum
+// with another -0 shows: a state that holds negative zeros may come out with
+// other signs of zero than from the scalar form, and with the same values.  A
+// multiply-add of -0, which keeps the sign, is fused like the product (kinetic
+// passes then differ in the last place).
 __device__ __forceinline__ float2 mul_(float2 a, float2 b) { return __ffma2_rn(a, b, make_float2(0.0f, 0.0f)); }
 __device__ __forceinline__ float2 fma_(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
 __device__ __forceinline__ float2 sub_(float2 a, float2 b) {
@@ -179,7 +184,7 @@ __device__ __forceinline__ void collide_pair_each(float2 (&d)[9], float2 (&g)[10
 // ---- the kinetic closures --------------------------------------------------
 // collide_xf, filtered_shift, carati_taus and the moment sums of
 // lbmhd_kinetic.cu (a file compiled without contraction) with every rounding
-// written out: the same operations in the same order, so the same bits.
+// written out: the same operations in the same order, so the same values.
 __device__ __forceinline__ float recip_(float v) { return __frcp_rn(v); }
 __device__ __forceinline__ float2 recip_(float2 v) { return make_float2(__frcp_rn(v.x), __frcp_rn(v.y)); }
 __device__ __forceinline__ float root_(float v) { return __fsqrt_rn(v); }

@@ -1,6 +1,7 @@
 // lbmhd_step_pipe.cu -- S = 2, 3 or 4 LB-MHD time steps in one pass over the
 // state, for the FP32 and FP16 storage forms with the local rates or no
-// closure (les 0, 1): the bits of S single steps (lbmhd_step.cu).
+// closure (les 0, 1): the values of S single steps (lbmhd_step.cu), bit for bit
+// but for the sign of a zero (mul_, lbmhd_pair.cuh).
 //
 // Why: the one-step kernel moves 152 B per node update (FP32) at the copy
 // bandwidth (1.03 of it at 8192^2), so only fewer passes over HBM make it
@@ -449,7 +450,7 @@ __global__ void __launch_bounds__(32, 4 * pipe_warps(sizeof(typename Fmt<P>::S),
 }
 
 // kPipeSteps steps of every run of an ensemble, a warp per strip-segment of a
-// run, so every run gets the bits of its own lattice.
+// run, so every run gets the values of its own lattice.
 template <int P, bool AL>
 __global__ void __launch_bounds__(32, 4 * batch_pipe_warps(sizeof(typename Fmt<P>::S)))
     batch_pipe_kernel(const RunDev<float>* runs, const RunPass* pass,

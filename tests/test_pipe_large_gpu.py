@@ -93,3 +93,28 @@ def test_narrow_and_flat_lattices_take_single_steps(L, prec, shape):
     got, launches = run(L, shape, prec, 1, (5,), False, fields=fields)
     ref, one = run(L, shape, prec, 1, (5,), True, fields=fields)
     assert np.array_equal(got, ref) and launches == one == 5
+
+
+@pytest.mark.parametrize("prec", ["fp32", "fp32_dev", "fp16_dev"])
+@pytest.mark.parametrize("les,shape", [(1, (128, 64)), (1, (57, 33)), (2, (1200, 1000)), (3, (1200, 1000))])
+def test_negative_zeros_change_no_value(L, prec, les, shape):
+    """A state with negative zeros, which the packed product does not keep: the
+    same values as single steps of one node per thread, and the same bits
+    wherever the value is not zero."""
+    nx, ny = shape
+    g = np.random.default_rng(2)
+    dev = np.where(g.random((19, ny, nx)) < 0.5, -0.0, 0.0)
+    dev[:, : ny // 2] += np.where(g.random((19, ny // 2, nx)) < 0.3, 0.0, g.normal(0, 0.01, (19, ny // 2, nx)))
+    if prec == "fp32":
+        dev[:9] += np.array([4 / 9] + [1 / 9] * 4 + [1 / 36] * 4)[:, None, None]
+    scale, dtype = {"fp32": (1, np.float32), "fp32_dev": (1, np.float32), "fp16_dev": (1024, np.float16)}[prec]
+    state = (dev * scale).astype(dtype)
+    fields = [np.ones((ny, nx))] + [np.zeros((ny, nx))] * 4
+    n = 4 if les == 1 else 2
+    got, launches = run(L, shape, prec, les, (n,), False, state, fields)
+    ref, one = run(L, shape, prec, les, (n,), True, state, fields)
+    assert (launches, one) == (1, n)
+    assert np.array_equal(got, ref)
+    bits = {2: np.uint16, 4: np.uint32}[got.dtype.itemsize]
+    other = np.ascontiguousarray(got).view(bits) != np.ascontiguousarray(ref).view(bits)
+    assert not np.any(got[other])
