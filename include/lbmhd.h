@@ -562,10 +562,13 @@ int lbmhd_batch_set_launch(lbmhd_batch_t* b, int vec, int block, int steps_per_l
 int lbmhd_batch_get_launch(const lbmhd_batch_t* b, int* vec, int* block, int* steps_per_launch);
 
 /* Autotuner: times every available (vec, block, steps_per_launch) for
- * trial_steps steps on a rest state and keeps the fastest.  Results are
- * cached in the JSON file cache_path (key: GPU name, precision, the
- * multiset of lattice shapes); a cached key is applied without timing.
- * The shape serves the steps that are not taken in passes of four.
+ * trial_steps steps on a rest state, and passes of four steps where the
+ * ensemble is one that they are for, and keeps the fastest.  Where that is
+ * the passes, the fastest shape serves the steps that are left over.
+ * Results are cached in the JSON file cache_path (key: GPU name, precision,
+ * the multiset of lattice shapes; value: the shape, the throughput of what
+ * was kept, and 1 if that is the passes, else 0); a cached key is applied
+ * without timing (four numbers: passes as lbmhd_batch_create would).
  * cache_path may be NULL (no cache).  Must run before any
  * lbmhd_batch_init (ESTATE otherwise); best_mlups (may be NULL) receives
  * the winner's throughput. */

@@ -464,7 +464,7 @@ std::map<std::string, std::vector<double>> load_cache(const std::string& path) {
             v.push_back(x);
             q = end;
         }
-        if (v.size() == 4) m[key] = v;
+        if (v.size() == 4 || v.size() == 5) m[key] = v;
         i = e + 1;
     }
     return m;
@@ -477,9 +477,10 @@ void save_cache(const std::string& path, const std::map<std::string, std::vector
     std::fprintf(f, "{\n");
     size_t k = 0;
     for (const auto& kv : m) {
-        std::fprintf(f, "  \"%s\": [%d, %d, %d, %.1f]%s\n", kv.first.c_str(), (int)kv.second[0],
-                     (int)kv.second[1], (int)kv.second[2], kv.second[3],
-                     ++k < m.size() ? "," : "");
+        std::fprintf(f, "  \"%s\": [%d, %d, %d, %.1f", kv.first.c_str(), (int)kv.second[0],
+                     (int)kv.second[1], (int)kv.second[2], kv.second[3]);
+        if (kv.second.size() > 4) std::fprintf(f, ", %d", (int)kv.second[4]);
+        std::fprintf(f, "]%s\n", ++k < m.size() ? "," : "");
     }
     std::fprintf(f, "}\n");
     std::fclose(f);
@@ -809,9 +810,10 @@ int lbmhd_batch_autotune(lbmhd_batch_t* b, const char* cache_path, int trial_ste
     if (trial_steps < 2) return bfail(LBMHD_EINVAL, "trial_steps must be >= 2");
     for (int r = 0; r < b->nruns; ++r)
         if (b->run_init[r]) return bfail(LBMHD_ESTATE, "autotune runs before lbmhd_batch_init");
-    // the shapes are those of the one-step kernel; ensembles that take several
-    // steps per pass do so whatever was set before
-    b->pipe = batch_pipe_ok(b);
+    // the shapes are those of the one-step kernel; passes of several steps are
+    // one more candidate, whatever was set before
+    const bool passes_ok = batch_pipe_ok(b);
+    b->pipe = passes_ok;
     const std::string key = tune_key(b);
     std::lock_guard<std::mutex> lock(g_tune_mu);
     std::map<std::string, std::vector<double>> cache;
@@ -819,12 +821,14 @@ int lbmhd_batch_autotune(lbmhd_batch_t* b, const char* cache_path, int trial_ste
         cache = load_cache(cache_path);
         auto it = cache.find(key);
         if (it != cache.end()) {
-            rc = set_shape(b, (int)it->second[0], (int)it->second[1],
-                                        (int)it->second[2]);
+            // four numbers (no word on passes): by the rule for ensembles
+            b->pipe = passes_ok && (it->second.size() < 5 || it->second[4] != 0.0);
+            rc = set_shape(b, (int)it->second[0], (int)it->second[1], (int)it->second[2]);
             if (rc == LBMHD_OK) {
                 if (best_mlups) *best_mlups = it->second[3];
                 return LBMHD_OK;
             }
+            b->pipe = passes_ok;
         }
     }
     // timing state: every run at rest (rho = 1, u = B = 0), built on device
@@ -882,30 +886,38 @@ int lbmhd_batch_autotune(lbmhd_batch_t* b, const char* cache_path, int trial_ste
                     bs = s;
                 }
             }
+    bool passes = false;
     if (use_pipe(b)) {
         LBMHD_BCK(b, launch_pass(b, b->cur));
         b->cur ^= 1;
-        LBMHD_BCK(b, cudaEventRecord(e0, b->stream));
-        const int passes = std::max(1, trial_steps / kPipeSteps);
-        for (int l = 0; l < passes; ++l) {
-            LBMHD_BCK(b, launch_pass(b, b->cur));
-            b->cur ^= 1;
+        const int n = std::max(2, trial_steps / kPipeSteps);
+        for (int rep = 0; rep < 3; ++rep) {
+            LBMHD_BCK(b, cudaEventRecord(e0, b->stream));
+            for (int l = 0; l < n; ++l) {
+                LBMHD_BCK(b, launch_pass(b, b->cur));
+                b->cur ^= 1;
+            }
+            LBMHD_BCK(b, cudaEventRecord(e1, b->stream));
+            LBMHD_BCK(b, cudaEventSynchronize(e1));
+            float ms = 0.f;
+            LBMHD_BCK(b, cudaEventElapsedTime(&ms, e0, e1));
+            const double mlups = (double)cells * n * kPipeSteps / (ms * 1e-3) / 1e6;
+            if (mlups > best) {
+                best = mlups;
+                passes = true;
+            }
         }
-        LBMHD_BCK(b, cudaEventRecord(e1, b->stream));
-        LBMHD_BCK(b, cudaEventSynchronize(e1));
-        float ms = 0.f;
-        LBMHD_BCK(b, cudaEventElapsedTime(&ms, e0, e1));
-        best = std::max(best, (double)cells * passes * kPipeSteps / (ms * 1e-3) / 1e6);
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     rc = read_batch_flag(b);
     if (rc) return rc;
+    b->pipe = passes;
     rc = set_shape(b, bv, bb, bs);
     if (rc) return rc;
     if (best_mlups) *best_mlups = best;
     if (cache_path && *cache_path) {
-        cache[key] = {(double)bv, (double)bb, (double)bs, best};
+        cache[key] = {(double)bv, (double)bb, (double)bs, best, passes ? 1.0 : 0.0};
         save_cache(cache_path, cache);
     }
     b->steps = 0;
