@@ -521,10 +521,11 @@ int lbmhd_diagnostics(lbmhd_t* h, lbmhd_diag* out) {
     if (!out) return fail(LBMHD_EINVAL, "out is NULL");
     if (!h->initialised) return fail(LBMHD_ESTATE, "diagnostics before lbmhd_init");
     DeviceGuard dg(h->device);
-    double v[13];  // and the flag
+    constexpr size_t kSums = 12 * sizeof(double);  // the flag follows them
+    double v[13];
     LBMHD_CK(h, launch_diag(h->p.precision, h->buf[h->cur], h->d_partials, h->d_diag, h->geom,
                             h->coll, h->stream));
-    LBMHD_CK(h, cudaMemcpyAsync(v, h->d_diag, sizeof(v), cudaMemcpyDeviceToHost, h->stream));
+    LBMHD_CK(h, cudaMemcpyAsync(v, h->d_diag, kSums + sizeof(int), cudaMemcpyDeviceToHost, h->stream));
     LBMHD_CK(h, cudaStreamSynchronize(h->stream));
     int flag;
     std::memcpy(&flag, v + 12, sizeof flag);
