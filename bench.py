@@ -9,7 +9,8 @@ A launch takes up to four steps in one pass over the state; the roofline
 fraction is that of a pass.  The state (5.1 GB per buffer) is far larger
 than L2, so no flush is needed between launches.  The same run also times,
 on the same lattice, the paper's kinetic LES (les = 2; two steps per pass,
-the fused one-step kernel and the two-pass kernels), the FP64, double-word (FF), FP32-deviation and FP16-deviation
+the fused one-step kernel and the two-pass kernels), the FP64, double-word
+(FF), FP32-deviation and FP16-deviation
 storage forms (fewer steps), an end-to-end pass through the host C ABI
 (host fields in, host moments out), the 256-run ensemble, the adjoint
 (gradients), and the CPU oracle on a bounded sample.

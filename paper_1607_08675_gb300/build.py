@@ -17,8 +17,9 @@ BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "liblbmhd.so")
 INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 
-SOURCES = ["lbmhd_step.cu", "lbmhd_step_pipe.cu", "lbmhd_step_tma.cu", "lbmhd_aux.cu", "lbmhd_runtime.cu", "lbmhd_noalloc.cu",
-           "lbmhd_batch.cu", "lbmhd_adjoint.cu", "lbmhd_kinetic.cu", "lbmhd3.cu"]
+SOURCES = ["lbmhd_step.cu", "lbmhd_step_pipe.cu", "lbmhd_step_tma.cu", "lbmhd_aux.cu",
+           "lbmhd_runtime.cu", "lbmhd_noalloc.cu", "lbmhd_batch.cu", "lbmhd_adjoint.cu",
+           "lbmhd_kinetic.cu", "lbmhd3.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2",
          "--expt-relaxed-constexpr", "-I", INCLUDE]
@@ -28,7 +29,7 @@ FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-Xcompiler", 
 # perform the same operations in the same order but in differently shaped
 # code, and only with every fusion written out is "same operations" also
 # "same bits".
-FILE_FLAGS = {"lbmhd_step_pipe.cu": ["-fmad=false"], "lbmhd_kinetic.cu": ["-fmad=false"], "lbmhd3.cu": ["-fmad=false"]}
+FILE_FLAGS = {f: ["-fmad=false"] for f in ("lbmhd_step_pipe.cu", "lbmhd_kinetic.cu", "lbmhd3.cu")}
 
 
 def nvcc() -> str:

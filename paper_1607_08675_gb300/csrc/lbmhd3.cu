@@ -1127,7 +1127,8 @@ __global__ void __launch_bounds__(256) step3_kernel(const typename Fmt3<P>::S* _
 // thread, leaving room for two CTAs of 128 threads per SM instead of three
 // (measured 14.1K against 16.8K MLUPS at 256^3).  Both nodes go through the
 // collision together in packed FP32: 17.6K MLUPS against 16.6K one after the
-// other (0.93 of the copy bandwidth at 360 B per node, from 0.89).
+// other (0.93 of the copy bandwidth at 360 B per node, from 0.89).  Bound by HBM
+// (ncu, 192^3: DRAM 78% with 31% of the issue slots busy).
 __global__ void __maxnreg__(168)
     step3f_kernel(const float* __restrict__ src, float* __restrict__ dst, Geom3 g, unsigned total,
                   unsigned total_pad, Coll3<float> c) {
@@ -1221,8 +1222,8 @@ __device__ __noinline__ void init3_node_f64(const double r, const double (&u)[3]
 
 // The same equilibria in double-word FP32 (FP32 and FP16 storage): false where
 // a value's rounding is not settled.  Directions c and -c share every even
-// term.  Error bound as in 2D: fewer than 40 operations of 2^-48, relative to
-// the sum m of the terms' magnitudes.
+// term.  Error bound as in 2D (init_node_ff): the longest path adds up to
+// 59 x 2^-48 of the sum m of the terms' magnitudes, twice that is used.
 template <int P>
 __device__ __forceinline__ bool init3_node_ff(double dr, const double (&du)[3], const double (&dB)[3],
                                               typename Fmt3<P>::S* __restrict__ st, long long i,
@@ -1360,9 +1361,11 @@ __device__ __noinline__ void moments3_node_odd(const typename Fmt3<P>::S* __rest
     moments3_node_f64<P>(st, ps, i, i16, m);
 }
 
-// The seven fields of every node.  FP32 and FP16 values sum exactly in FP64 in
-// any order: line, plane and volume sums (75 FP64 operations against about
-// 250), widened by moving bits, and one reciprocal.
+// The seven fields of every node.  FP32 and FP16: line, plane and volume sums
+// (75 FP64 operations against about 250) of values widened by moving bits, and
+// one reciprocal.  A sum of 27 24-bit values is exact in FP64 whatever its order
+// while their exponents lie within 24 bits, and else within a few 2^-53 of the
+// sum of their magnitudes, as in any order.
 template <int P>
 __global__ void moments3_kernel(const typename Fmt3<P>::S* __restrict__ st, long long ps,
                                 long long n, Fields7 out, double i16) {

@@ -234,11 +234,13 @@ __device__ __forceinline__ void collide_adjoint(const R (&d)[9], const R (&g)[10
 namespace {
 
 constexpr int kAdjBlock = 256;
-// At most the two resident blocks per SM of a 152-SM GB300 (114 registers): each
-// thread sweeps its share of the nodes, so the final reduction of the
-// sensitivity sums, whose FP64 additions hold a scheduler's pipe for 64 clocks
-// each, is paid once per resident thread (us per adjoint step, four waves of
-// blocks / one: FP32 512^2 29.2 / 12.8, 2048^2 163.6 / 158.8).
+// At most two blocks per SM of a 152-SM GB300: each thread sweeps its share of
+// the nodes, so the final reduction of the sensitivity sums, whose FP64
+// additions hold a scheduler's pipe for 64 clocks each, is paid once per thread.
+// FP32 and FP32_DEV hold both at once (113 and 114 registers), one wave; FP64 and
+// FF (160, 173) hold one and run two waves.  us per adjoint step, eight blocks
+// per SM / two: FP32 512^2 29.2 / 12.8, 2048^2 163.6 / 158.8; a whole backward step
+// with its recomputed one, 512^2: FP64 345 / 303, FF 112 / 92.
 constexpr int kAdjMaxBlocks = 2 * 152;
 
 __device__ __forceinline__ int wrapi(int a, int n) { return a < 0 ? a + n : (a >= n ? a - n : a); }

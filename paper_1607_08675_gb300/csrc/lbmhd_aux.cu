@@ -80,8 +80,10 @@ __device__ __noinline__ void init_node_f64(double r, double u, double v, double 
 
 // The same equilibria in double-word FP32, for the FP32 and FP16 forms.  False
 // where a value's rounding is not settled (nothing to rely on was stored).
-// Error bound: fewer than 40 operations of 2^-48 each on the way to a value,
-// relative to the sum m of its terms' magnitudes, so 2^-41 m w.
+// Error bound, relative to the sum m of a value's terms' magnitudes: a product
+// is good to 6 x 2^-48, a sum to 4 x 2^-48, a product by an FP32 constant to
+// 3 x 2^-48, an input to 2^-49; the longest path adds up to 47 x 2^-48, and
+// 2^-41 m w, nearly three times that, is used.
 template <int P>
 __device__ __forceinline__ bool init_node_ff(double dr, double du, double dv, double dX, double dY,
                                              typename Fmt<P>::S* __restrict__ st, long long c,
@@ -188,10 +190,11 @@ __device__ __noinline__ void node_moments_odd(const typename Fmt<P>::S* __restri
     node_moments_f64<P>(st, ps, o, inv_scale, m);
 }
 
-// The FP32 and FP16 forms: sums of 24-bit values are exact in FP64, so their
-// order is free -- shared pair sums, the weights subtracted once, the FP16
-// scale applied to the sums, and the values widened by moving bits: 34 FP64
-// operations (42 for FP16) instead of about 85.
+// The FP32 and FP16 forms: shared pair sums, the weights subtracted once, the
+// FP16 scale applied to the sums, and the values widened by moving bits: 34
+// FP64 operations (42 for FP16) instead of about 85.  A sum of ten 24-bit values
+// is exact in FP64 whatever its order while their exponents lie within 25 bits,
+// and else within a few 2^-53 of the sum of their magnitudes, as in any order.
 template <int P>
 __device__ __forceinline__ void node_moments(const typename Fmt<P>::S* __restrict__ st,
                                              long long ps, long long o, float inv_scale,

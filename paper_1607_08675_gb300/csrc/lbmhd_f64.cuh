@@ -18,6 +18,7 @@
 //    they differ from the IEEE ones in an occasional last place.  Operands
 //    outside the range of the FP32 start, 2^-120 to 2^120, take the IEEE ones.
 // Every operation is rounded as written, so all kernels give the same bits.
+// ncu, 2048^2, one node per thread: the FP64 pipe 86% busy, issue 10%, DRAM 13%.
 // Measured (GB300, us per step, collide() / this, one node per thread):
 // 1024^2 399.5 / 295.4, 256^2 28.7 / 21.6, 64^2 8.5 / 6.6.
 #pragma once

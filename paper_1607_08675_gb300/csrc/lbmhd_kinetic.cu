@@ -8,7 +8,7 @@
 //     into every node (pull + sums) into five planes;
 //  2. step_kin_kernel: per node, pull the populations, take central
 //     differences of those planes at x +- 1, y +- 1, form the corrections
-//     (filtered_shift) and collide (collide<..., KIN>) -- or, for les = 3,
+//     (filtered_shift) and collide (collide_xf<..., KIN>) -- or, for les = 3,
 //     the closure's relaxation times (carati_taus) and collide with them.
 // One node per thread; neighbouring threads share the moment loads in L1.
 // The default is a fused one-pass kernel (below) with the same arithmetic;

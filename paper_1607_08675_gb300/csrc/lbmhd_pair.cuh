@@ -5,12 +5,12 @@
 //
 // Both come from the one source below, and every FP32 step kernel calls it, so
 // they give the same values whatever shape the compiler gives their code, bit
-// for bit but for the sign of a zero (see mul_).  The
-// operations are those of collide() (lbmhd_device.cuh) with its products fused
-// into the sums that follow.  ABS: FP32 storage of the populations themselves
-// fuses the second product of j_x j_y / rho - B_x B_y instead of the first.  A
-// sign moved from a term to a constant (n8, the outputs, -1/tau_m) changes no
-// rounding.
+// for bit but for the sign of a zero (see mul_).  The operations are those of
+// collide() (lbmhd_device.cuh) with its products fused into the sums that
+// follow.  ABS: FP32 storage of the populations themselves fuses the second
+// product of j_x j_y / rho - B_x B_y instead of the first; neither is the more
+// accurate, and each keeps the results that its format had.  A sign moved from
+// a term to a constant (n8, the outputs, -1/tau_m) changes no rounding.
 #pragma once
 
 #include <type_traits>

@@ -13,9 +13,9 @@ constexpr int pipe_halo(int S) { return (S + 1) / 2 * 2; }
 constexpr int pipe_useful(int S) { return (64 - pipe_halo(S) - S) / 2 * 2; }
 
 // Warps per scheduler that the registers are cut for (65536 / 128 / warps);
-// `bytes` of a stored value.  4 bytes: 128 registers at S = 2, 168 at S = 3, 255
-// at S = 4 (three warps spill there: 72 G); 2 bytes, whose history is packed,
-// 128 at every S.
+// `bytes` of a stored value.  4 bytes: 116 registers at S = 2, 156 at S = 3, 208
+// at S = 4 (242 with odd rows; three warps spill there: 72 G); 2 bytes, whose
+// history is packed, at most 128 at every S.
 constexpr int pipe_warps(int bytes, int S) { return bytes == 2 || S == 2 ? 4 : (S == 3 ? 3 : 2); }
 // An ensemble's run rates are read by every lane into registers.
 constexpr int batch_pipe_warps(int bytes) { return bytes == 2 ? 3 : 2; }

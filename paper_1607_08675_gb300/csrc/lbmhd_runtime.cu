@@ -268,13 +268,13 @@ int lbmhd_create(int nx, int ny, const lbmhd_params* p, lbmhd_t** out) {
     // 6.0 / 5.4, 8192 x 64 10.1 / 8.8, 2048^2 98.7 / 95.9, 8192^2 1467 / 1463, the
     // copy bandwidth).  FP16 storage: eight nodes (16-byte loads) in 32-thread
     // blocks, 82.0K MLUPS at 8192^2, but four in 64-thread blocks up to 2^20 - 1
-    // nodes (512^2 5.0 / 4.2, 768^2 7.6 / 7.4, 1024^2 12.5 / 12.8).  FP64 is bound by the FP64 pipe, and one node per
-    // thread in 64-thread blocks spreads it best at every size (us per step, two
-    // nodes in 128-thread blocks / this: 64^2 13.2 / 6.6, 256^2 24.4 / 21.6,
-    // 1024^2 303.9 / 295.4).  Double-word FF: two nodes in 256-thread blocks,
-    // but one in 128-thread blocks where the lattice leaves SMs idle (64^2 7.3 /
-    // 3.9, 256^2 8.0 / 6.8, 512^2 22.7 / 20.5, 768^2 51.5 / 52.1).  Narrower
-    // vectors when nx is not a multiple.
+    // nodes (512^2 5.0 / 4.2, 768^2 7.6 / 7.4, 1024^2 12.5 / 12.8).  FP64 is bound
+    // by the FP64 pipe, and one node per thread in 64-thread blocks spreads it
+    // best at every size (us per step, two nodes in 128-thread blocks / this:
+    // 64^2 13.2 / 6.6, 256^2 24.4 / 21.6, 1024^2 303.9 / 295.4).  Double-word FF:
+    // two nodes in 256-thread blocks, but one in 128-thread blocks where the
+    // lattice leaves SMs idle (64^2 7.3 / 3.9, 256^2 8.0 / 6.8, 512^2 22.7 / 20.5,
+    // 768^2 51.5 / 52.1).  Narrower vectors when nx is not a multiple.
     const bool ff_small = p->precision == LBMHD_FF && (long long)nx * ny <= 1LL << 18;
     const int want = p->precision == LBMHD_FP64 || ff_small
                          ? 1

@@ -27,10 +27,13 @@
 // own wait orders it).  The two columns of a lane go through the collision
 // together in packed two-wide FP32 instructions (lbmhd_pair.cuh).
 //
-// Bound: instruction issue (177 instructions per update and thread at
-// S = 3, 47% of the issue slots and 51% of the FMA pipe busy) with the
-// latency of few warps: the history of S - 1 steps takes registers, two to
-// four warps per scheduler.  Measured on GB300, 8192^2, updates per second:
+// Bound: instruction issue and the FMA pipe with the latency of few warps: the
+// history of S - 1 steps takes registers, two to four warps per scheduler.  ncu,
+// 4096^2, S = 4: FP32 173 instructions per update and thread, 54% of the issue
+// slots and 61% of the FMA pipe busy, 60% of DRAM, 1.1 cycles per instruction
+// waiting for a fixed latency and none of the others above 0.4; FP16 194
+// instructions, 63% and 65%, 31% of DRAM, 1.4 cycles waiting for the pipe.
+// Measured on GB300, 8192^2, updates per second:
 //   FP32  one-step 45.9 G;  S = 2 82.6 G;  S = 3 121.5 G;  S = 4 127.9 G
 //   FP16  one-step 81.6 G;  S = 2 124 G;   S = 3 132 G;    S = 4 133.9 G
 // and 1024^2 (FP32) 36.9 -> 93.0 G, 1999 x 1201 (odd rows) 34.3 -> 95.6 G.
@@ -277,7 +280,9 @@ __device__ __forceinline__ void pipe_body(const typename Fmt<P>::S* __restrict__
 // 8192^2 FP32 les 2 1735 / 1116, les 3 1737 / 1098; FP16 les 2 1521 / 1081, les 3
 // 1517 / 955; 4096^2 FP32 les 2 448 / 293.  The one-step kernel ran at 0.87 of
 // the copy bandwidth at 152 B per node; this one is bound by issue and
-// latency at two warps per scheduler.
+// latency at two warps per scheduler (ncu, 4096^2 FP32 les 2: 353 instructions
+// per update and thread, 52% of the issue slots, 56% of the FMA pipe, 56% of
+// DRAM).
 template <int P, bool AL>
 struct KinShared {
     using Q = typename PairOf<P>::T;
@@ -450,7 +455,8 @@ __global__ void __launch_bounds__(32, 4 * pipe_warps(sizeof(typename Fmt<P>::S),
 }
 
 // kPipeSteps steps of every run of an ensemble, a warp per strip-segment of a
-// run, so every run gets the values of its own lattice.
+// run, so every run gets the values of its own lattice.  Bound as above (ncu, 64
+// runs of 512^2 FP32: 54% of the issue slots, 56% of the FMA pipe, 50% of DRAM).
 template <int P, bool AL>
 __global__ void __launch_bounds__(32, 4 * batch_pipe_warps(sizeof(typename Fmt<P>::S)))
     batch_pipe_kernel(const RunDev<float>* runs, const RunPass* pass,
