@@ -41,7 +41,7 @@ struct PipePlan {
 // The length is the best by the mean unless that leaves the busiest scheduler
 // more than 1/6 above the least, as where a few schedulers get one warp more:
 // then it is the best by the busiest.  FP32, us per step, the mean's length /
-// the busiest's: 1024 x 585 10.1 / 8.0, 256 x 2343 11.2 / 8.4; within the 1/6,
+// the busiest's: 1024 x 585 10.1 / 7.7, 256 x 2343 11.2 / 7.6; within the 1/6,
 // 1024^2 (19 / 16 rows) 12.3 / 11.0 for one run but 10.20 / 10.38 for two at once.
 template <class Units>
 PipePlan pipe_plan(int S, int warps, int most, int sm_count, Units units_of) {
@@ -80,7 +80,7 @@ PipePlan pipe_plan(int S, int warps, int most, int sm_count, Units units_of) {
 // and the one-step kernel falls to the rate of HBM; or up to 32768 nodes, where
 // a launch is mostly latency and one for four steps takes less than four.
 // Between them the rows that segments share cost as much as the passes save
-// (FP32, us per step, one-step / pass: 512^2 5.8 / 6.3).
+// (FP32, us per step, one-step / pass: 512^2 5.2 / 6.3).
 constexpr long long kPipeBytes = 80LL << 20;
 constexpr long long kPipeSmall = 32768;
 
@@ -106,8 +106,8 @@ inline double one_step_us(int bytes, long long nodes, int align, bool ensemble) 
 // one, or the runs of an ensemble).  A strip computes 64 columns whatever the
 // lattice has, and rows around a segment whatever its rows, so this depends on
 // the shape, not on the nodes alone (GB300, us per step, one-step / pass, FP32
-// 2^21 nodes in rows of 8, 16, 24, 64 and 256: 48 / 122, 48 / 60, 48 / 43,
-// 48 / 33, 48 / 20; in 1, 2 and 4 rows 48 / 70, 47 / 44, 47 / 32).
+// 2^21 nodes in rows of 8, 16, 24, 64 and 256: 48 / 122, 48 / 60, 48 / 40,
+// 48 / 31, 48 / 20; in 1, 2 and 4 rows 48 / 70, 47 / 44, 47 / 32).
 //
 // Large: by the plan's time and that of four single steps.  Of 430 lattices
 // and ensembles timed, none takes a pass that is more than 2% slower and none
@@ -147,8 +147,8 @@ inline bool pipe_pays(int bytes, int nruns, const int* nx, const int* ny, bool e
 }
 
 // The kinetic closures, two steps per pass: only the large ones (les 2 FP32, us
-// per step, one-step / pass: 128^2 2.9 / 3.6, 512^2 11.4 / 12.2, 1024^2 39.4 /
-// 25.6).  Their one-step kernel sweeps strips of 256 columns, so narrow lattices
+// per step, one-step / pass: 128^2 3.0 / 3.6, 512^2 11.6 / 12.2, 1024^2 36.1 /
+// 26.3).  Their one-step kernel sweeps strips of 256 columns, so narrow lattices
 // gain the most (2^21 nodes in rows of 2, 16, 57, 113 and 256: 2015 / 1868, 347 /
 // 131, 126 / 84, 86 / 65, 67 / 44); rows fewer than four are slower in a pass
 // (1, 2, 3 rows: 76 / 143, 68 / 93, 69 / 76).

@@ -3,7 +3,7 @@
 
 The segment length must leave the busiest scheduler at most 1/6 above the least.
 Measured on GB300 (152 SMs, us per step, a length that gives a few schedulers
-one warp more / this): FP32 1024 x 585 10.1 / 8.0, 256 x 2343 11.2 / 8.4.
+one warp more / this): FP32 1024 x 585 10.1 / 7.7, 256 x 2343 11.2 / 7.6.
 """
 import os
 import shutil
